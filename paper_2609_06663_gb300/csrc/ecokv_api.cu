@@ -36,7 +36,7 @@ Layout make_layout(const ecokv_params& p, int nrec) {
   const size_t U = (size_t)L.U;
   size_t off = 0;
   L.status = off;  off += 256;
-  L.sync = off;    L.sync_bytes = (4 + 2 * U) * 4;  off += align256(L.sync_bytes);
+  L.sync = off;    L.sync_bytes = (4 + U) * 4;  off += align256(L.sync_bytes);
   L.p1part = off;  off += align256(U * L.nchunks * L.p1_stride * 4);
   L.ustat = off;   off += align256(U * L.ustat_stride * 4);
   L.p2part = off;  off += align256(U * L.nchunks * kP2Stride * 4);
@@ -79,7 +79,7 @@ static int tc_group_rows(int R) { return (R + tc_groups(R) - 1) / tc_groups(R); 
 static bool use_tensor_path(const ecokv_params& p, ecokv_dtype dt) {
   if (dt != ECOKV_BF16 || (p.flags & ECOKV_FLAG_FORCE_SIMT)) return false;
   if (p.n < 128) return false;
-  return tc_rows_half(tc_group_rows((p.h_q / p.h_kv) * p.window)) > 0;
+  return tc_rows(tc_group_rows((p.h_q / p.h_kv) * p.window)) > 0;
 }
 
 // Stage events of this host thread (ecokv_set_stage_events), recorded on the
@@ -106,10 +106,8 @@ static int tc_wave_units(const ecokv_params& p) {
 // Record slots per unit of the tensor-core passes (a bound over grids of up
 // to kTcMaxSms CTAs, so that it does not depend on the device).
 static int tc_records(const ecokv_params& p) {
-  const long long U = (long long)p.n_layers * p.h_kv;
-  const int T = (p.n + 127) / 128, uw = tc_wave_units(p);
-  const long long nw = (U + uw - 1) / uw, last = U - (nw - 1) * uw;
-  return tc_record_slots(T, (int)((uw < last ? uw : last) * T));
+  const int T = (p.n + 127) / 128;
+  return tc_record_slots(T, (int)(tc_wave_units(p) * T));
 }
 
 // SMs of the current device (cached per device).
@@ -234,7 +232,7 @@ static ecokv_status run_tc_group(const ecokv_params& p, const Layout& L, const v
   a.R = rows;
   a.R4 = (rows + 3) & ~3;
   a.row0 = row0;
-  a.NP = 2 * tc_rows_half(rows_max);
+  a.RP = tc_rows(rows_max);
   a.g = p.h_q / p.h_kv;
   a.h_kv = p.h_kv;
   a.h_q = p.h_q;
@@ -248,6 +246,7 @@ static ecokv_status run_tc_group(const ecokv_params& p, const Layout& L, const v
   if (a.lag > a.nw) a.lag = a.nw;
   const int sms = num_sms();
   a.P = sms < kTcMaxSms ? sms : kTcMaxSms;
+  a.smin = a.uw * a.T / a.P > 1 ? a.uw * a.T / a.P : 1;
   a.rmax = L.nchunks;
   a.p1_stride = L.p1_stride;
   a.ustat_stride = L.ustat_stride;

@@ -1,0 +1,43 @@
+"""The tensor-core kernel's instances by window rows: the smallest and largest
+row count of each (its padding rows, the columns read at once, two or three
+tile groups), over slices of several tiles with a ragged end, against the fp64
+oracle."""
+import pytest
+import torch
+
+from oracle import ecokv_oracle as O
+from paper_2609_06663_gb300 import ecokv as E
+from paper_2609_06663_gb300.workloads import make_inputs, small_workload
+from tests.parity import TOL, check_scores, check_selection, oracle_params
+from tests.test_gpu_parity import params_of, run_and_compare
+
+pytestmark = pytest.mark.gpu
+
+
+# g x W window rows: instances of 8, 16, 32, 56, 64, 112 and 128 rows
+@pytest.mark.parametrize("group,window", [(1, 1), (1, 8), (3, 3), (2, 8), (1, 17), (4, 8), (3, 11), (7, 8), (3, 19),
+                                          (8, 8), (5, 13), (7, 16), (1, 113), (8, 15)],
+                         ids=lambda v: str(v))
+def test_window_row_instances(group, window):
+    # 470 tiles of one head: three or four a CTA, so that every tile group
+    # works and pass 2 walks back over more than one tile
+    run_and_compare(small_workload(60001, h_kv=1, group=group, window=window, budget=6000, dtype="bf16", seed=2))
+
+
+@pytest.mark.parametrize("group,window", [(1, 8), (7, 8), (7, 16)], ids=lambda v: str(v))
+def test_logits_that_outgrow_their_reference(group, window):
+    """Keys that grow along the sequence: the logits of a slice's later tiles
+    exceed the first key's by far more than 2^6, so that the reference of the
+    partial sums has to be raised, several times over."""
+    w = small_workload(60000, h_kv=1, group=group, window=window, budget=6000, dtype="bf16", seed=4)
+    K, V, Q = make_inputs(w)
+    ramp = torch.linspace(0.2, 30.0, 128).repeat((w.n + 127) // 128)[:w.n]
+    tile = torch.arange(w.n) // 128 % 4
+    K = (K.float() * (ramp * (1.0 + tile))[None, None, :, None]).to(torch.bfloat16)
+    p = params_of(w)
+    op = oracle_params(p)
+    idx, _, _, S, lam = E.evict(p, K.cuda(), V.cuda(), Q.cuda(), want_scores=True)
+    r = O.evict(K, V, Q, op)[(0, 0)]
+    check_scores(S[0, 0].cpu().double().numpy(), r, TOL["bf16"], "growing keys")
+    check_selection(idx[0, 0].cpu().numpy(), r, op, TOL["bf16"], "growing keys")
+    assert abs(float(lam[0, 0]) - r["lam"]) <= TOL["bf16"]
