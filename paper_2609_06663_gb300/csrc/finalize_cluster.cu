@@ -3,11 +3,12 @@
 // (finalize_select.cuh), spread over the cluster so that every SM takes part,
 // with the cluster-wide reductions done through distributed shared memory.
 //
-// Two shapes: 16 candidates a thread and up to 8 CTAs (units up to 32768
-// candidates, used up to 16384), or 32 candidates a thread and up to 4 CTAs
-// (units of 16385 to 32768): at four CTAs per SM the GPU holds about 74
-// clusters of 8 but 148 of 4, so the long units of a prefill (e.g. 28 layers
-// x 4 KV heads of 32k tokens) run in one wave instead of one and a half.
+// Shapes: 8, 16 or 32 candidates a thread and up to 4 CTAs (units of up to
+// 8192, 16384 and 32768 candidates), or 32 a thread and up to 16 CTAs (up to
+// 131072).  Four CTAs a unit at the most where that is enough: at three or
+// more CTAs per SM the 112 units of a prefill (28 layers x 4 KV heads) are
+// then resident in one wave (clusters of 8 would need one and a half), and the
+// kernel, all latency, takes one unit's time.
 //
 // CTA rank r of the cluster owns candidates [r * cap, (r + 1) * cap) of the
 // unit (cap = 256 threads x kJ); thread t of it owns the kJ consecutive
@@ -22,17 +23,26 @@
 //      S_div over the cluster;
 //   3. S (Eq. 7) as finalize_unit computes it, divisions by the min-max
 //      ranges and the pooling kernel taken as reciprocal products;
-//   4. MSB-first radix select over the order-preserving image of S, one
-//      256-bin histogram per CTA, summed over the cluster for each 8-bit digit;
-//   5. counts of keys above / equal to the threshold, scanned over the
-//      threads and exchanged between the CTAs, so that each thread knows how
-//      many kept candidates precede its own (ties to the lower position);
+//   4. the k-th largest key: one histogram over kBins equal ranges of the
+//      keys' order-preserving images between bounds of S, summed over the
+//      cluster, finds the range that holds it; the keys in that range (of a
+//      long unit about a hundred) are gathered by every CTA and ranked
+//      directly.  A range that holds more than kList keys is split again, a
+//      range of one value (ties) is the answer;
+//   5. the kept candidates ahead of each thread's own (ties to the lower
+//      position), from the same histograms, lists and a scan over the threads;
 //      then its kept positions in ascending order (the last CTA adds the
 //      window).  The gather of the kept rows is its own launch.
 // Cluster barriers are reached by every CTA on every path (no early exit).
 // Every exchange between CTAs is a store into the peers' shared memory
 // (each CTA keeps every rank's contribution) followed by a cluster barrier,
 // so no CTA waits on a remote load.
+//
+// What bounds it: the chain of barriers and L2 round trips of one unit (no
+// HBM traffic of its own): from the streaming grid's end 10 us for 8 units of
+// 1020 candidates, 14 us for 4 of 4995, 28 us for 112 of 32760 (slowest CTA).
+// With an 8-bit radix select of four digits, each a cluster exchange, and the
+// distances loaded only once their extrema were known: 19, 20 and 35 us.
 
 #include <atomic>
 
@@ -49,45 +59,50 @@ constexpr int kCThreads = 256;
 constexpr int kCWarps = kCThreads / 32;
 constexpr int kHalo = 16;  // pooling halo kept in shared memory (kernel <= 33)
 
-// Shapes (kSh): 0 = 16 candidates a thread, up to 8 CTAs; 1 = 32 a thread,
-// up to 4 CTAs; 2 = 32 a thread, up to 16 CTAs (clusters past the portable 8,
-// for units of 32769 to 131072 candidates; their larger exchange buffers
-// would cost the 4-CTA shape occupancy).
+// Shapes (kSh), see above: candidates a thread, CTAs a unit, histogram ranges
+// (their 16-bit counts of every rank take the place of the staged scores).
 template <int kSh>
 struct Shape {
-  static constexpr int kJ = kSh == 0 ? 16 : 32;                            // candidates a thread owns
-  static constexpr int kCap = kCThreads * kJ;                              // candidates a CTA owns
-  static constexpr int kMaxCluster = kSh == 0 ? 8 : (kSh == 1 ? 4 : 16);  // CTAs a unit may take
-  static constexpr int kQ = kCap + 2 * kHalo;                              // staged raw votes
+  static constexpr int kJ = kSh == 0 ? 8 : (kSh == 1 ? 16 : 32);  // candidates a thread owns
+  static constexpr int kCap = kCThreads * kJ;                     // candidates a CTA owns
+  static constexpr int kMaxCluster = kSh == 3 ? 16 : 4;           // CTAs a unit may take
+  static constexpr int kQ = kCap + 2 * kHalo;                     // staged raw votes
+  static constexpr int kBins = kSh == 1 || kSh == 2 ? 2048 : 1024;
+  static constexpr int kMinCtas = kSh == 1 ? 3 : 4;               // resident CTAs per SM asked of the compiler
 };
+constexpr int kList = 512;  // keys ranked directly
 
 // Padded shared-memory index of staged position q.
 __device__ __forceinline__ int pad_idx(int q) { return q + (q >> 5); }
 
 template <int kSh>
 struct ClusterSmem {
-  // raw vote of candidate lo - kHalo + q at raw[pad_idx(q)]
-  float raw[Shape<kSh>::kQ + Shape<kSh>::kQ / 32 + 1];
-  unsigned whist[kCWarps][256];  // per radix pass, each warp's own histogram
-  // Written by the peers (distributed shared memory stores): per radix pass
-  // the histogram of every rank (double-buffered across passes), the S_div
-  // extrema and the counts above / equal to the threshold of every rank.
-  unsigned hall[2][Shape<kSh>::kMaxCluster][256];
-  float ext_all[Shape<kSh>::kMaxCluster][2];
-  double simp_all[Shape<kSh>::kMaxCluster];  // value-norm importance: every rank's sum of S_imp
-  double wsum_all[Shape<kSh>::kMaxCluster];  // winsorised min-max / MAD scaling: every rank's sum of s_E terms
-  int cnt_all[Shape<kSh>::kMaxCluster][2];
+  using Sh = Shape<kSh>;
+  union {
+    // raw vote of candidate lo - kHalo + q at raw[pad_idx(q)]; S_div and the scores later
+    float raw[Sh::kQ + Sh::kQ / 32 + 1];
+    // then, written by the peers: every rank's histogram
+    alignas(16) uint16_t hall[Sh::kMaxCluster][Sh::kBins];
+  };
+  alignas(16) unsigned hist[Sh::kBins];
+  // Written by the peers (distributed shared memory stores): the extrema of
+  // S_div and of S_imp (of the keys, when the scores are given), and the keys
+  // in the range of the k-th largest.
+  alignas(16) unsigned list[kList + 4];
+  float4 ext_all[Sh::kMaxCluster];
+  double simp_all[Sh::kMaxCluster];  // value-norm importance: every rank's sum of S_imp
+  double wsum_all[Sh::kMaxCluster];  // winsorised min-max / MAD scaling: every rank's sum of s_E terms
   float red[kCWarps][8];  // per-warp partials
+  float4 red4[kCWarps];   // per-warp extrema
   float edge[32];         // pooling edge values
   float sc[8];            // broadcast scalars
   double dsc[2];          // sums behind the means of S_imp and of S_div
   double dred[kCWarps];   // per-warp sums of S_imp (value-norm importance)
   double dredw[kCWarps];  // per-warp sums of the clipped d_E (winsorised min-max) or of s_E (MAD scaling)
-  float wmax;             // winsorised min-max: the upper clip bound
-  float mmed, minv;       // MAD scaling: the median of d_E and 1 / (MAD + eps)
   unsigned wsum[kCWarps];
-  int wscan[kCWarps][2];  // per-warp counts above / equal to the threshold
+  alignas(16) int wscan[kCWarps][4];  // per-warp counts above / equal to the threshold, and of lower ranks' keys
   int shi[4];
+  unsigned lcount;        // keys this CTA has put on the list
 };
 
 // Composite diversity (Eq. 2 and Eq. 3) with the min-max divisor applied as a
@@ -105,12 +120,20 @@ __device__ __forceinline__ float mad_logistic(float dE, float med, float inv) {
   return 1.f / (1.f + expf(-__fmul_rn(__fsub_rn(dE, med), inv)));
 }
 
-// Store v into the same object of every CTA of the cluster (its own included).
-template <int kMaxC, typename T>
-__device__ __forceinline__ void push_all(cg::cluster_group& cl, T* obj, T v, int C) {
-#pragma unroll
-  for (int r = 0; r < kMaxC; ++r)
-    if (r < C) *cl.map_shared_rank(obj, r) = v;
+// Barrier over the cluster (a block barrier when the unit has one CTA), whole
+// or as its two halves.
+__device__ __forceinline__ void unit_arrive(int C) {
+  if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void unit_wait(int C) {
+  if (C > 1)
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  else
+    __syncthreads();
+}
+__device__ __forceinline__ void unit_sync(int C) {
+  unit_arrive(C);
+  unit_wait(C);
 }
 
 // kMode: 0 = scores, 1 = scores and top-k, 2 = top-k of given scores (f.S).
@@ -118,9 +141,9 @@ __device__ __forceinline__ void push_all(cg::cluster_group& cl, T* obj, T v, int
 // variants are compiled in (their code is left out of the default kernel, whose register budget it
 // would cost).
 template <int kMode, int kSh, bool kVar>
-__global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArgs f) {
+__global__ void __launch_bounds__(kCThreads, Shape<kSh>::kMinCtas) finalize_cluster_kernel(FinalArgs f) {
   constexpr bool kSelect = kMode != 0;
-  constexpr int kJ = Shape<kSh>::kJ, kCap = Shape<kSh>::kCap, kMaxC = Shape<kSh>::kMaxCluster;
+  constexpr int kJ = Shape<kSh>::kJ, kCap = Shape<kSh>::kCap;
   extern __shared__ __align__(16) uint8_t fc_smem[];
   ClusterSmem<kSh>& sm = *reinterpret_cast<ClusterSmem<kSh>*>(fc_smem);
   cg::cluster_group cl = cg::this_cluster();
@@ -155,6 +178,7 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
 
   // pooled importance (as float bits), then the order-preserving keys of S
   unsigned key[kJ];
+  unsigned klo = 0u, khi = 0xffffffffu;  // bounds of the keys (the first histogram's range; none need hold)
 
   if (kMode == 2) {
     // scores given (absent when nothing is to be chosen): staged in
@@ -167,11 +191,65 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
         if (i < Tv) sm.raw[pad_idx(i - lo + kHalo)] = __ldg(Su + i);
       }
       __syncthreads();
+      unsigned mnk = 0xffffffffu, mxk = 0u;
 #pragma unroll
-      for (int c = 0; c < kJ; ++c) key[c] = ordered_key(sm.raw[pad_idx(q0 + c)]);
+      for (int c = 0; c < kJ; ++c) {
+        key[c] = ordered_key(sm.raw[pad_idx(q0 + c)]);
+        if (c < nv) {
+          mnk = min(mnk, key[c]);
+          mxk = max(mxk, key[c]);
+        }
+      }
+      mnk = __reduce_min_sync(0xffffffffu, mnk);
+      mxk = __reduce_max_sync(0xffffffffu, mxk);
+      if (lane == 0) {
+        sm.red[warp][0] = __uint_as_float(mnk);
+        sm.red[warp][1] = __uint_as_float(mxk);
+      }
+      __syncthreads();
+      asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+      if (tid < C) {
+        unsigned a0 = __float_as_uint(sm.red[0][0]), a1 = __float_as_uint(sm.red[0][1]);
+        for (int w = 1; w < kCWarps; ++w) {
+          a0 = min(a0, __float_as_uint(sm.red[w][0]));
+          a1 = max(a1, __float_as_uint(sm.red[w][1]));
+        }
+        *cl.map_shared_rank(&sm.ext_all[rank], tid) =
+            make_float4(__uint_as_float(a0), __uint_as_float(a1), 0.f, 0.f);
+      }
+      unit_sync(C);
+      klo = 0xffffffffu;
+      khi = 0u;
+      for (int r = 0; r < C; ++r) {
+        klo = min(klo, __float_as_uint(sm.ext_all[r].x));
+        khi = max(khi, __float_as_uint(sm.ext_all[r].y));
+      }
+    } else {
+      asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     }
-    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   } else {
+    // the distances and cosines of the CTA's candidates (for step 2; with 32
+    // candidates a thread they do not fit the registers and are read there)
+    constexpr bool kEarly = kJ <= 16;
+    constexpr int kBatch = kEarly ? kJ / 4 : 4;  // groups of four whose loads are in flight together
+    const float* dEu = f.dE + (size_t)u * Tv;
+    const float* cvu = f.cosv + (size_t)u * Tv;
+    float4 ea[kBatch], ca[kBatch];
+    // groups of four from the (kBatch b0)-th on, this thread's in coalesced
+    // order; a group not wholly below Tv is left to the scalar loop
+    auto load_batch = [&](int b0) {
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j) {
+        const int i = lo + 4 * (kCThreads * (b0 + j) + tid);
+        ea[j] = ca[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i + 3 < Tv) {
+          ea[j] = __ldg(reinterpret_cast<const float4*>(dEu + i));
+          ca[j] = __ldg(reinterpret_cast<const float4*>(cvu + i));
+        }
+      }
+    };
+    if (kEarly && vec4) load_batch(0);
+
     // 1. the six pass-2 partials (sum over all N of d_E, min / max / sum of
     //    d_E, sums of cosines and of raw votes over the candidates); meanwhile
     //    the CTA's raw votes with the pooling halo and the edge values
@@ -263,44 +341,46 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
         }
       }
     }
-    if (tid == 0) {
-      float s_all = sm.red[0][0], mnE = sm.red[0][1], mxE = sm.red[0][2];
-      float s_de = sm.red[0][3], s_c = sm.red[0][4], s_raw = sm.red[0][5];
-      for (int w = 1; w < kCWarps; ++w) {
-        s_all += sm.red[w][0];
-        mnE = fminf(mnE, sm.red[w][1]);
-        mxE = fmaxf(mxE, sm.red[w][2]);
-        s_de += sm.red[w][3];
-        s_c += sm.red[w][4];
-        s_raw += sm.red[w][5];
-      }
-      if (kVar && f.wlo != nullptr) {  // winsorised min-max: the order statistics replace the extrema
-        mnE = key_float(f.wlo[4 * u]);
-        mxE = key_float(f.whi[4 * u]);
-      }
-      sm.wmax = mxE;
-      sm.sc[0] = s_all;
-      sm.sc[1] = mnE;
-      sm.sc[2] = __fadd_rn(__fsub_rn(mxE, mnE), f.eps);
-      if (kVar && f.mad != nullptr) {
-        // MAD scaling: the sweep maps d_E to s_E itself, so the affine map
-        // that follows it is the identity
-        const int nu = f.n_units;
-        const float lo2 = key_float(f.mad[4 * u]), hi2 = key_float(f.mad[4 * (nu + u)]);
-        const float dlo = key_float(f.mad[4 * (2 * nu + u)]), dhi = key_float(f.mad[4 * (3 * nu + u)]);
-        sm.mmed = __fmul_rn(0.5f, __fadd_rn(lo2, hi2));
-        sm.minv = 1.f / __fadd_rn(__fmul_rn(0.5f, __fadd_rn(dlo, dhi)), f.eps);
-        sm.sc[1] = 0.f;
-        sm.sc[2] = 1.f;
-      }
-      sm.sc[3] = s_de;
-      sm.sc[4] = s_c;
-      sm.sc[5] = s_raw;
+    // every thread takes the extrema of d_E from the warps' partials
+    float mnE = sm.red[0][1], wmax = sm.red[0][2];
+#pragma unroll
+    for (int w = 1; w < kCWarps; ++w) {
+      mnE = fminf(mnE, sm.red[w][1]);
+      wmax = fmaxf(wmax, sm.red[w][2]);
     }
-    // (this barrier also ends every thread's reads of the staged raw votes)
-    __syncthreads();
-    const float mnE = sm.sc[1], denE = sm.sc[2];
+    if (kVar && f.wlo != nullptr) {  // winsorised min-max: the order statistics replace the extrema
+      mnE = key_float(f.wlo[4 * u]);
+      wmax = key_float(f.whi[4 * u]);
+    }
+    float denE = __fadd_rn(__fsub_rn(wmax, mnE), f.eps);
+    float mmed = 0.f, minv = 0.f;
+    if (kVar && f.mad != nullptr) {
+      // MAD scaling: the sweep maps d_E to s_E itself, so the affine map
+      // that follows it is the identity
+      const int nu = f.n_units;
+      const float lo2 = key_float(f.mad[4 * u]), hi2 = key_float(f.mad[4 * (nu + u)]);
+      const float dlo = key_float(f.mad[4 * (2 * nu + u)]), dhi = key_float(f.mad[4 * (3 * nu + u)]);
+      mmed = __fmul_rn(0.5f, __fadd_rn(lo2, hi2));
+      minv = 1.f / __fadd_rn(__fmul_rn(0.5f, __fadd_rn(dlo, dhi)), f.eps);
+      mnE = 0.f;
+      denE = 1.f;
+    }
     const float invE = __frcp_rn(denE);
+    // extrema of the pooled importance (for the bounds of the keys; not negative, so ordered as integers)
+    float mnI, mxI;
+    auto imp_extrema = [&]() {
+      unsigned a = 0x7f800000u, b = 0u;
+#pragma unroll
+      for (int c = 0; c < kJ; ++c)
+        if (c < nv) {
+          a = min(a, key[c]);
+          b = max(b, key[c]);
+        }
+      mnI = __uint_as_float(__reduce_min_sync(0xffffffffu, a));
+      mxI = __uint_as_float(__reduce_max_sync(0xffffffffu, b));
+    };
+    // the threads' reads of the staged raw votes end here
+    __syncthreads();
     if (kVar && f.vnorm != nullptr) {
       // value-norm importance: S_imp = pooled vote * ||v||, the norms staged
       // in coalesced order where the raw votes were; the sum of S_imp (its
@@ -327,13 +407,17 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
       if (lane == 0) sm.dred[warp] = ps;
       __syncthreads();  // also: every norm read before the S_div sweep reuses the buffer
     }
+    if (kSelect) imp_extrema();
 
+    // Unit scalars, while the other threads compute S_div: one warp's lane
+    // each, so that no warp's share holds up the next barrier.
     if (tid == 32) {
-      // off the critical path, while the other threads compute S_div:
       // per-head redundancy and lambda (Eq. 4-6) in single precision (lambda
       // weighs two terms of order one: its rounding stays at the level of the
-      // scores' own), and the parts of the means that need no cluster extremum
-      const float D_E = __fdiv_rn(sm.sc[0], (float)f.N);
+      // scores' own)
+      float s_all = sm.red[0][0];
+      for (int w = 1; w < kCWarps; ++w) s_all += sm.red[w][0];
+      const float D_E = __fdiv_rn(s_all, (float)f.N);
       const float tau = f.tau > 0.f ? f.tau : sqrtf((float)kD);
       const float r_E = 2.f - 2.f / (1.f + expf(-D_E / tau));
       const float mu_sq = __ldg(us + ustat_musq());
@@ -342,10 +426,11 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
       if (f.flags & ECOKV_FLAG_LAMBDA_OVERRIDE) lam = f.lambda_override;
       if (f.lambda != nullptr && rank == 0) f.lambda[u] = lam;
       sm.sc[0] = lam;
+    } else if (tid == 64) {
       // means, in double and scaled by Tv: sum_i S_imp(i) = (1/kp) sum_j
-      // raw(j) cnt(j), where cnt(j) = kp except within kp/2 of either end;
-      // mean(Sbar) is affine in the means of d_E and of the cosine (as
-      // finalize_unit)
+      // raw(j) cnt(j), where cnt(j) = kp except within kp/2 of either end
+      float s_raw = sm.red[0][5];
+      for (int w = 1; w < kCWarps; ++w) s_raw += sm.red[w][5];
       const int h = hpool;
       double edge = 0.0;
       if (pool_smem) {
@@ -357,11 +442,19 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
         for (int j = 0; j < Tv && j < h; ++j) edge += (double)__ldg(raw + j) * (double)(h - j);
         for (int j = (Tv - h > 0 ? Tv - h : 0); j < Tv; ++j) edge += (double)__ldg(raw + j) * (double)(h - (Tv - 1 - j));
       }
+      sm.dsc[0] = (double)f.pool * (double)s_raw - edge;  // kp * Tv * mean(S_imp)
+    } else if (tid == 96) {
+      // mean(Sbar) is affine in the means of d_E and of the cosine (as finalize_unit)
+      float s_de = sm.red[0][3], s_c = sm.red[0][4];
+      for (int w = 1; w < kCWarps; ++w) {
+        s_de += sm.red[w][3];
+        s_c += sm.red[w][4];
+      }
       const double T = (double)Tv;
-      const double sum_sE = ((double)sm.sc[3] - (double)mnE * T) / (double)denE;
-      const double sum_cs = (double)sm.sc[4];
+      const double sum_sE = ((double)s_de - (double)mnE * T) / (double)denE;
+      const double sum_cs = (double)s_c;
       const double sum_sC = mix ? -sum_cs : (T - sum_cs) * 0.5;
-      sm.dsc[0] = (double)f.pool * (double)sm.sc[5] - edge;                      // kp * Tv * mean(S_imp)
+      sm.sc[4] = s_c;
       sm.dsc[1] = (double)f.alpha * sum_sE + (1.0 - (double)f.alpha) * sum_sC;  // Tv * mean(S_div)
     }
 
@@ -371,68 +464,43 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
     float mnD = INFINITY, mxD = -INFINITY;
     const bool wins = kVar && f.wlo != nullptr;
     const bool madv = kVar && f.mad != nullptr;
-    const float wmax = sm.wmax, mmed = sm.mmed, minv = sm.minv;
     // this thread's sum of the clipped d_E (winsorised min-max) or of s_E (MAD
     // scaling): at most 32 terms in single precision, the reductions in double
     float wsumf = 0.f;
-    {
-      const float* dEu = f.dE + (size_t)u * Tv;
-      const float* cvu = f.cosv + (size_t)u * Tv;
-      if (vec4) {
-  #pragma unroll 4
-        for (int j = 0; j < kJ / 4; ++j) {
-          const int i = lo + 4 * (kCThreads * j + tid);
-          if (i < Tv) {
-            float e[4] = {0.f, 0.f, 0.f, 0.f}, cs[4] = {0.f, 0.f, 0.f, 0.f};
-            if (i + 3 < Tv) {
-              const float4 a4 = __ldg(reinterpret_cast<const float4*>(dEu + i));
-              const float4 b4 = __ldg(reinterpret_cast<const float4*>(cvu + i));
-              e[0] = a4.x; e[1] = a4.y; e[2] = a4.z; e[3] = a4.w;
-              cs[0] = b4.x; cs[1] = b4.y; cs[2] = b4.z; cs[3] = b4.w;
-            } else {
-              for (int r = 0; r < 4 && i + r < Tv; ++r) {
-                e[r] = __ldg(dEu + i + r);
-                cs[r] = __ldg(cvu + i + r);
-              }
-            }
-  #pragma unroll
-            for (int r = 0; r < 4; ++r)
-              if (i + r < Tv) {
-                if (wins) {
-                  e[r] = fminf(fmaxf(e[r], mnE), wmax);
-                  wsumf = __fadd_rn(wsumf, e[r]);
-                } else if (madv) {
-                  e[r] = mad_logistic(e[r], mmed, minv);
-                  wsumf = __fadd_rn(wsumf, e[r]);
-                }
-                const float sd = sdiv_rcp(e[r], cs[r], mnE, invE, f.alpha, mix);
-                sm.raw[pad_idx(i + r - lo + kHalo)] = sd;
-                mnD = fminf(mnD, sd);
-                mxD = fmaxf(mxD, sd);
-              }
-          }
-        }
-      } else {
-  #pragma unroll 8
-        for (int j = 0; j < kJ; ++j) {
-          const int i = lo + kCThreads * j + tid;
-          if (i < Tv) {
-            float e = __ldg(dEu + i);
-            if (wins) {
-              e = fminf(fmaxf(e, mnE), wmax);
-              wsumf = __fadd_rn(wsumf, e);
-            } else if (madv) {
-              e = mad_logistic(e, mmed, minv);
-              wsumf = __fadd_rn(wsumf, e);
-            }
-            const float sd = sdiv_rcp(e, __ldg(cvu + i), mnE, invE, f.alpha, mix);
-            sm.raw[pad_idx(i - lo + kHalo)] = sd;
-            mnD = fminf(mnD, sd);
-            mxD = fmaxf(mxD, sd);
+    auto sweep1 = [&](int i, float e, float cs) {
+      if (wins) {
+        e = fminf(fmaxf(e, mnE), wmax);
+        wsumf = __fadd_rn(wsumf, e);
+      } else if (madv) {
+        e = mad_logistic(e, mmed, minv);
+        wsumf = __fadd_rn(wsumf, e);
+      }
+      const float sd = sdiv_rcp(e, cs, mnE, invE, f.alpha, mix);
+      sm.raw[pad_idx(i - lo + kHalo)] = sd;
+      mnD = fminf(mnD, sd);
+      mxD = fmaxf(mxD, sd);
+    };
+    const int hi = min(Tv, lo + kCap);  // candidates of this CTA: [lo, hi)
+    int tail = lo;                      // the scalar loop's first
+    if (vec4) {
+      tail = max(lo, hi & ~3);
+#pragma unroll
+      for (int b0 = 0; b0 < kJ / 4; b0 += kBatch) {
+        if (!kEarly) load_batch(b0);
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+          const int i = lo + 4 * (kCThreads * (b0 + j) + tid);
+          if (i + 3 < Tv) {
+            sweep1(i, ea[j].x, ca[j].x);
+            sweep1(i + 1, ea[j].y, ca[j].y);
+            sweep1(i + 2, ea[j].z, ca[j].z);
+            sweep1(i + 3, ea[j].w, ca[j].w);
           }
         }
       }
     }
+#pragma unroll 8
+    for (int i = tail + tid; i < hi; i += kCThreads) sweep1(i, __ldg(dEu + i), __ldg(cvu + i));
     if (wins || madv) {
       double wsum = (double)wsumf;
   #pragma unroll
@@ -444,38 +512,41 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
       mnD = fminf(mnD, __shfl_xor_sync(0xffffffffu, mnD, o));
       mxD = fmaxf(mxD, __shfl_xor_sync(0xffffffffu, mxD, o));
     }
-    if (lane == 0) {
-      sm.red[warp][6] = mnD;
-      sm.red[warp][7] = mxD;
-    }
+    if (lane == 0) sm.red4[warp] = make_float4(mnD, mxD, kSelect ? mnI : 0.f, kSelect ? mxI : 0.f);
     __syncthreads();
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-    if (tid == 0) {
-      float a0 = sm.red[0][6], a1 = sm.red[0][7];
+    if (tid < C) {  // one thread a peer
+      float4 a = sm.red4[0];
+#pragma unroll
       for (int w = 1; w < kCWarps; ++w) {
-        a0 = fminf(a0, sm.red[w][6]);
-        a1 = fmaxf(a1, sm.red[w][7]);
+        const float4 b = sm.red4[w];
+        a = make_float4(fminf(a.x, b.x), fmaxf(a.y, b.y), fminf(a.z, b.z), fmaxf(a.w, b.w));
       }
-      push_all<kMaxC>(cl, &sm.ext_all[rank][0], a0, C);
-      push_all<kMaxC>(cl, &sm.ext_all[rank][1], a1, C);
+      *cl.map_shared_rank(&sm.ext_all[rank], tid) = a;
       if (kVar && f.vnorm != nullptr) {
         double cs = 0.0;
         for (int w = 0; w < kCWarps; ++w) cs += sm.dred[w];
-        push_all<kMaxC>(cl, &sm.simp_all[rank], cs, C);
+        *cl.map_shared_rank(&sm.simp_all[rank], tid) = cs;
       }
       if (wins || madv) {
         double cs = 0.0;
         for (int w = 0; w < kCWarps; ++w) cs += sm.dredw[w];
-        push_all<kMaxC>(cl, &sm.wsum_all[rank], cs, C);
+        *cl.map_shared_rank(&sm.wsum_all[rank], tid) = cs;
       }
     }
-    cl.sync();
+    unit_sync(C);
     if (tid == 0) {
       float a0 = INFINITY, a1 = -INFINITY;
+      float i0 = INFINITY, i1 = 0.f;
       for (int r = 0; r < C; ++r) {
-        a0 = fminf(a0, sm.ext_all[r][0]);
-        a1 = fmaxf(a1, sm.ext_all[r][1]);
+        const float4 e = sm.ext_all[r];
+        a0 = fminf(a0, e.x);
+        a1 = fmaxf(a1, e.y);
+        i0 = fminf(i0, e.z);
+        i1 = fmaxf(i1, e.w);
       }
+      sm.sc[1] = i0;
+      sm.sc[2] = i1;
       const float denD = __fadd_rn(__fsub_rn(a1, a0), f.eps);
       // mean(S_imp) / mean(Sbar) with Sbar = (S_div - a0) / denD
       double dsc1 = sm.dsc[1];  // Tv * mean(S_div)
@@ -502,6 +573,12 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
     const float lamf = sm.sc[0], mnD2 = sm.sc[6], denD = sm.sc[7], scale = sm.sc[5];
     const float invD = __frcp_rn(denD);
     const float one_m_lam = __fsub_rn(1.f, lamf);
+    if (kSelect) {
+      // bounds of S: Sbar lies in [0, 1], S_imp between its extrema
+      const float i0 = sm.sc[1], i1 = sm.sc[2], d1 = lamf * scale;
+      klo = ordered_key(fminf(0.f, d1) + fminf(one_m_lam * i0, one_m_lam * i1));
+      khi = ordered_key(fmaxf(0.f, d1) + fmaxf(one_m_lam * i0, one_m_lam * i1));
+    }
 
     // 3. final scores (Eq. 7); the keys replace the pooled importance, and
     //    the scores go out through the staging buffer in coalesced order
@@ -518,8 +595,6 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
       // cosine, S_div, recomputed by the same operations (kept out of the
       // loop above, whose code size sets its speed)
       float* dbg = f.dbg + (size_t)u * 5 * Tv;
-      const float* dEu = f.dE + (size_t)u * Tv;
-      const float* cvu = f.cosv + (size_t)u * Tv;
       const float inv_pool = __frcp_rn((float)f.pool);
   #pragma unroll 1
       for (int c = 0; c < nv; ++c) {
@@ -562,49 +637,60 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
   }
 
   if (kSelect) {
-    // 4. radix select of the k-th largest key over the cluster
-    unsigned prefix = 0u, mask = 0u;
-    int rem = k;
+    // 4. the k-th largest key
+    unsigned thr = 0u;
+    int rem = k;               // keys still to take from the range [klo, khi]
+    int gt_low = 0, eq_low = 0;  // this thread's share of the lower ranks' keys above / equal to thr
+    constexpr int kBins = Shape<kSh>::kBins, kPer = kBins / kCThreads;  // ranges a thread sums
     if (k > 0) {
-      int pass = 0;
-      for (int shift = 24; shift >= 0; shift -= 8, ++pass) {
-        // each warp counts into its own histogram, a thread adding runs of
-        // equal bins among its consecutive candidates (neighbouring scores
-        // share their leading bits), then the CTA's histogram is the sum of
-        // its warps'
-        unsigned* wh = sm.whist[warp];
+      for (bool first = true;; first = false) {
+        // kBins ranges of 2^shift keys from klo on; on the first pass klo and
+        // khi are estimates: keys outside fall into the end ranges
+        const unsigned span = khi > klo ? khi - klo : 0u;
+        const int shift = max(0, 32 - __clz(span) - (kBins == 2048 ? 11 : 10));
 #pragma unroll
-        for (int b = lane; b < 256; b += 32) wh[b] = 0u;
-        __syncwarp();
-        unsigned cur = 0u, run = 0u;
+        for (int b = 0; b < kPer; b += 4) *reinterpret_cast<uint4*>(&sm.hist[kPer * tid + b]) = make_uint4(0u, 0u, 0u, 0u);
+        if (tid == 0) sm.lcount = 0u;
+        __syncthreads();
 #pragma unroll
-        for (int c = 0; c < kJ; ++c) {
-          if (c < nv && (key[c] & mask) == prefix) {
-            const unsigned bin = (key[c] >> shift) & 255u;
-            if (bin != cur) {
-              if (run) atomicAdd(&wh[cur], run);
-              cur = bin;
-              run = 0u;
-            }
-            ++run;
+        for (int c = 0; c < kJ; ++c)
+          if (c < nv && (first || (key[c] >= klo && key[c] <= khi))) {
+            const unsigned d = key[c] > klo ? (key[c] - klo) >> shift : 0u;
+            atomicAdd(&sm.hist[min(d, (unsigned)kBins - 1u)], 1u);
+          }
+        // no thread of the cluster reads its raw / hall any more once all have arrived
+        unit_arrive(C);
+        __syncthreads();
+        unit_wait(C);
+        {
+          uint32_t pk[kPer / 2];  // counts of at most 8192 keys
+#pragma unroll
+          for (int b = 0; b < kPer; b += 2) pk[b / 2] = sm.hist[kPer * tid + b] | sm.hist[kPer * tid + b + 1] << 16;
+          for (int r = 0; r < C; ++r) {
+            uint16_t* dst = cl.map_shared_rank(&sm.hall[rank][kPer * tid], r);
+            if constexpr (kPer == 8)
+              *reinterpret_cast<uint4*>(dst) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            else
+              *reinterpret_cast<uint2*>(dst) = make_uint2(pk[0], pk[1]);
           }
         }
-        if (run) atomicAdd(&wh[cur], run);
-        __syncthreads();
-        {
-          unsigned cnt = 0u;  // kCThreads == 256 bins: thread tid sums bin tid
+        unit_sync(C);
+        // the cluster's histogram: this thread's ranges, then suffix sums
+        // from the top range find the one holding the rem-th largest key
+        unsigned h[kPer], tot = 0u;
 #pragma unroll
-          for (int w = 0; w < kCWarps; ++w) cnt += sm.whist[w][tid];
-          push_all<kMaxC>(cl, &sm.hall[pass & 1][rank][tid], cnt, C);
+        for (int b = 0; b < kPer; ++b) h[b] = 0u;
+        for (int r = 0; r < C; ++r) {
+#pragma unroll
+          for (int b = 0; b < kPer; b += 2) {
+            const uint32_t v = *reinterpret_cast<const uint32_t*>(&sm.hall[r][kPer * tid + b]);
+            h[b] += v & 0xffffu;
+            h[b + 1] += v >> 16;
+          }
         }
-        cl.sync();
-        // the cluster's histogram (rank order: deterministic), bin tid; suffix
-        // sums from the top bin find the bin holding the rem-th largest key
-        unsigned tot = 0u;
 #pragma unroll
-        for (int r = 0; r < kMaxC; ++r)
-          if (r < C) tot += sm.hall[pass & 1][r][tid];
-        unsigned suf = tot;  // sum of bins tid .. 32 * warp + 31
+        for (int b = 0; b < kPer; ++b) tot += h[b];
+        unsigned suf = tot;  // keys of threads tid .. 32 * warp + 31
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           const unsigned y = __shfl_down_sync(0xffffffffu, suf, o);
@@ -612,34 +698,114 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
         }
         if (lane == 0) sm.wsum[warp] = suf;
         __syncthreads();
-        for (int w = warp + 1; w < kCWarps; ++w) suf += sm.wsum[w];
-        // suf = keys in bins >= tid; the wanted bin has suf >= rem > suf - tot
+#pragma unroll
+        for (int w = 0; w < kCWarps; ++w)
+          if (w > warp) suf += sm.wsum[w];
         if (suf >= (unsigned)rem && suf - tot < (unsigned)rem) {
-          sm.shi[1] = tid;
-          sm.shi[2] = rem - (int)(suf - tot);
+          unsigned above = suf - tot;
+          bool found = false;
+#pragma unroll
+          for (int b = kPer - 1; b >= 0; --b) {
+            if (!found && above + h[b] >= (unsigned)rem) {
+              found = true;
+              sm.shi[0] = kPer * tid + b;
+              sm.shi[1] = rem - (int)above;
+              sm.shi[2] = (int)h[b];
+            }
+            if (!found) above += h[b];
+          }
         }
         __syncthreads();
-        prefix |= (unsigned)sm.shi[1] << shift;
-        mask |= 255u << shift;
-        rem = sm.shi[2];
-        // (the next write of shi follows the next pass's first barrier, which
-        // every thread reaches only after reading this one)
+        const unsigned sel = (unsigned)sm.shi[0];
+        rem = sm.shi[1];
+        const int cnt = sm.shi[2];
+        int before = 0;  // lower ranks' keys in the range
+        for (int r = 0; r < rank; ++r) {
+          before += sm.hall[r][sel];
+#pragma unroll
+          for (int b = 0; b < kPer; b += 2) {
+            const uint32_t v = *reinterpret_cast<const uint32_t*>(&sm.hall[r][kPer * tid + b]);
+            if ((unsigned)(kPer * tid + b) > sel) gt_low += (int)(v & 0xffffu);
+            if ((unsigned)(kPer * tid + b + 1) > sel) gt_low += (int)(v >> 16);
+          }
+        }
+        // the range, as wide as its keys may be
+        const unsigned rlo = klo + (sel << shift);
+        const unsigned rhi = rlo + ((1u << shift) - 1u);
+        if (first) {
+          klo = sel == 0u ? 0u : rlo;
+          khi = sel == (unsigned)kBins - 1u || rhi < rlo ? 0xffffffffu : rhi;
+        } else {
+          klo = rlo;
+          khi = rhi < rlo ? khi : min(khi, rhi);
+        }
+        if (klo == khi) {  // one value: ties
+          thr = klo;
+          if (tid == 0) eq_low = before;
+          break;
+        }
+        if (cnt <= kList) {
+          // every CTA gets the range's keys, rank by rank; each is ranked by
+          // counting (the keys of one rank come in any order: only their
+          // values are used)
+#pragma unroll
+          for (int c = 0; c < kJ; ++c)
+            if (c < nv && key[c] >= klo && key[c] <= khi) sm.hist[atomicAdd(&sm.lcount, 1u)] = key[c];
+          __syncthreads();
+          for (unsigned t = tid; t < sm.lcount; t += kCThreads)
+            for (int r = 0; r < C; ++r) *cl.map_shared_rank(&sm.list[before + t], r) = sm.hist[t];
+          if (tid < 3) sm.list[min(cnt + tid, kList + 2)] = 0u;  // the last group of four: below every key
+          unit_sync(C);
+          // 2^sp threads a key, each comparing it with every 2^sp-th group of four
+          const int sp = cnt <= 32 ? 3 : (cnt <= 64 ? 2 : (cnt <= 128 ? 1 : 0));
+          const int seg = tid & ((1 << sp) - 1);
+          for (int t0 = 0; t0 < cnt; t0 += kCThreads >> sp) {
+            const int t = t0 + (tid >> sp);
+            const unsigned x = sm.list[min(t, cnt - 1)];
+            int g = 0, e = 0;
+#pragma unroll 4
+            for (int i = 4 * seg; i < cnt; i += 4 << sp) {
+              const uint4 y = *reinterpret_cast<const uint4*>(&sm.list[i]);
+              g += (y.x > x) + (y.y > x) + (y.z > x) + (y.w > x);
+              e += (y.x == x) + (y.y == x) + (y.z == x) + (y.w == x);
+            }
+            for (int o = 1; o < 1 << sp; o <<= 1) {
+              g += __shfl_xor_sync(0xffffffffu, g, o);
+              e += __shfl_xor_sync(0xffffffffu, e, o);
+            }
+            if (t < cnt && g < rem && rem <= g + e) {  // the same for every key equal to it
+              sm.wsum[0] = x;
+              sm.wsum[1] = (unsigned)(rem - g);
+            }
+          }
+          __syncthreads();
+          thr = sm.wsum[0];
+          rem = (int)sm.wsum[1];
+          for (int t = tid; t < before; t += kCThreads) {
+            gt_low += sm.list[t] > thr;
+            eq_low += sm.list[t] == thr;
+          }
+          break;
+        }
       }
     }
-    const unsigned thr = prefix;
 
     // 5. kept candidates: above the threshold, or equal to it among the first
     //    `rem` equal ones by position, emitted in ascending position
-    int n_gt = 0, n_eq = 0;
+    unsigned m_gt = 0u, m_eq = 0u;  // a bit for each of this thread's candidates
     if (k > 0) {
 #pragma unroll
-      for (int c = 0; c < kJ; ++c)
-        if (c < nv) {
-          n_gt += key[c] > thr;
-          n_eq += key[c] == thr;
-        }
+      for (int c = 0; c < kJ; ++c) {
+        m_gt |= (key[c] > thr ? 1u : 0u) << c;
+        m_eq |= (key[c] == thr ? 1u : 0u) << c;
+      }
+      const unsigned have = nv >= 32 ? 0xffffffffu : (1u << nv) - 1u;
+      m_gt &= have;
+      m_eq &= have;
     }
-    // exclusive prefix over the threads of the CTA (position order)
+    const int n_gt = __popc(m_gt), n_eq = __popc(m_eq);
+    // exclusive prefix over the threads of the CTA (position order), and the
+    // lower ranks' counts
     int gi = n_gt, ei = n_eq;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -649,52 +815,37 @@ __global__ void __launch_bounds__(kCThreads, 4) finalize_cluster_kernel(FinalArg
         ei += ye;
       }
     }
+    gt_low = __reduce_add_sync(0xffffffffu, gt_low);
+    eq_low = __reduce_add_sync(0xffffffffu, eq_low);
     if (lane == 31) {
       sm.wscan[warp][0] = gi;
       sm.wscan[warp][1] = ei;
+      sm.wscan[warp][2] = gt_low;
+      sm.wscan[warp][3] = eq_low;
     }
     __syncthreads();
-    int gt_excl = gi - n_gt, eq_excl = ei - n_eq;
-    for (int w = 0; w < warp; ++w) {
-      gt_excl += sm.wscan[w][0];
-      eq_excl += sm.wscan[w][1];
-    }
-    if (tid == 0) {
-      int g = 0, q = 0;
-      for (int w = 0; w < kCWarps; ++w) {
-        g += sm.wscan[w][0];
-        q += sm.wscan[w][1];
+    int gt_excl = gi - n_gt, eq_excl = ei - n_eq, pos = 0, eq_before = 0;
+#pragma unroll
+    for (int w = 0; w < kCWarps; ++w) {
+      const int4 v = *reinterpret_cast<const int4*>(sm.wscan[w]);
+      if (w < warp) {
+        gt_excl += v.x;
+        eq_excl += v.y;
       }
-      push_all<kMaxC>(cl, &sm.cnt_all[rank][0], g, C);
-      push_all<kMaxC>(cl, &sm.cnt_all[rank][1], q, C);
+      pos += v.z;
+      eq_before += v.w;
     }
-    cl.sync();
-    // candidates kept by lower ranks, and the ties they took
-    int pos = 0, eq_before = 0;
-    for (int r = 0; r < rank; ++r) {
-      const int g = sm.cnt_all[r][0], q = sm.cnt_all[r][1];
-      pos += g + max(0, min(q, rem - eq_before));
-      eq_before += q;
-    }
-    // ties still to take from this CTA on, in position order
+    // candidates kept by lower ranks, and the ties still to take from this
+    // CTA on, in position order
+    pos += min(eq_before, rem);
     const int ties = max(0, rem - eq_before);
     int p = pos + gt_excl + min(ties, eq_excl);
-    int take_eq = max(0, min(n_eq, ties - eq_excl));
+    const int take_eq = max(0, min(n_eq, ties - eq_excl));
     int32_t* out = f.idx + (size_t)u * f.n_keep;
-    if (k > 0) {
-#pragma unroll
-      for (int c = 0; c < kJ; ++c)
-        if (c < nv) {
-          bool take = key[c] > thr;
-          if (!take && key[c] == thr && take_eq > 0) {
-            take = true;
-            --take_eq;
-          }
-          if (take) {
-            if (p < k) out[p] = c0 + c;
-            ++p;
-          }
-        }
+    while (__popc(m_eq) > take_eq) m_eq &= ~(0x80000000u >> __clz(m_eq));  // the first take_eq of them
+    for (unsigned m = m_gt | m_eq; m != 0u; m &= m - 1u) {
+      if (p < k) out[p] = c0 + __ffs(m) - 1;
+      ++p;
     }
     if (keep_all) {
       // B >= N: every row in order; rank r writes its candidates, the last rank the window
@@ -756,7 +907,7 @@ cudaError_t launch_shape(const FinalArgs& f, int U, int C, bool select_only, cud
 }
 
 // Per device: the attributes set, and whether clusters of 16 CTAs of the
-// long shape can be resident (cudaOccupancyMaxActiveClusters > 0).
+// longest shape can be resident (cudaOccupancyMaxActiveClusters > 0).
 std::atomic<int> g_setup[64];  // 0 = not yet, 1 = set, clusters of 16 unavailable, 2 = set and available
 
 int device_setup() {
@@ -764,13 +915,13 @@ int device_setup() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
   int st = g_setup[dev].load();
   if (st != 0) return st;
-  if (set_attrs<0>() != cudaSuccess || set_attrs<1>() != cudaSuccess) return -1;
+  if (set_attrs<0>() != cudaSuccess || set_attrs<1>() != cudaSuccess || set_attrs<2>() != cudaSuccess) return -1;
   st = 1;
-  if (set_attrs<2>() == cudaSuccess) {
+  if (set_attrs<3>() == cudaSuccess) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(16u * 16u, 1, 1);
     cfg.blockDim = dim3(kCThreads, 1, 1);
-    cfg.dynamicSmemBytes = sizeof(ClusterSmem<2>);
+    cfg.dynamicSmemBytes = sizeof(ClusterSmem<3>);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 16;
@@ -779,7 +930,7 @@ int device_setup() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (const void*)finalize_cluster_kernel<1, 2, false>, &cfg) == cudaSuccess &&
+    if (cudaOccupancyMaxActiveClusters(&n, (const void*)finalize_cluster_kernel<1, 3, false>, &cfg) == cudaSuccess &&
         n > 0)
       st = 2;
   }
@@ -788,25 +939,19 @@ int device_setup() {
   return st;
 }
 
-// Shape and cluster size for units of Tv candidates; shape -1 when no cluster
-// shape takes them.
+// Shape and cluster size for units of Tv candidates: the shortest shape whose
+// cluster takes them; shape -1 when none does.
 void pick_shape(int Tv, int long_ok, int& sh, int& C) {
   const int t = Tv > 0 ? Tv : 1;
-  const int C16 = (t + Shape<0>::kCap - 1) / Shape<0>::kCap;
-  const int C32 = (t + Shape<1>::kCap - 1) / Shape<1>::kCap;
-  if (C16 <= 4) {
-    sh = 0;
-    C = C16;
-  } else if (C32 <= Shape<1>::kMaxCluster) {
-    sh = 1;
-    C = C32;
-  } else if (C32 <= (long_ok ? Shape<2>::kMaxCluster : 8)) {
-    sh = 2;
-    C = C32;
-  } else {
-    sh = -1;
-    C = 0;
+  const int cap[4] = {Shape<0>::kCap, Shape<1>::kCap, Shape<2>::kCap, Shape<3>::kCap};
+  const int most[4] = {Shape<0>::kMaxCluster, Shape<1>::kMaxCluster, Shape<2>::kMaxCluster,
+                       long_ok ? Shape<3>::kMaxCluster : 8};
+  for (sh = 0; sh < 4; ++sh) {
+    C = (t + cap[sh] - 1) / cap[sh];
+    if (C <= most[sh]) return;
   }
+  sh = -1;
+  C = 0;
 }
 
 }  // namespace
@@ -828,6 +973,7 @@ cudaError_t launch_finalize_cluster(const FinalArgs& f, int U, bool select_only,
     case 0: return launch_shape<0>(f, U, C, select_only, s);
     case 1: return launch_shape<1>(f, U, C, select_only, s);
     case 2: return launch_shape<2>(f, U, C, select_only, s);
+    case 3: return launch_shape<3>(f, U, C, select_only, s);
   }
   return cudaErrorNotSupported;
 }
