@@ -98,11 +98,26 @@ def row_groups(w) -> int:
     return (w.group * w.window + 119) // 120
 
 
+SMS = 152  # of a GB300
+
+
+def short_units(w) -> bool:
+    """Few short heads take one launch for both passes, scores and selection:
+    up to 40 tiles of 128 keys and 64 window rows, one cluster per head, all
+    clusters (at most five tiles a CTA) on the GPU at once."""
+    tiles = (w.n + 127) // 128
+    ctas = min(8, tiles, SMS // w.units)
+    return tensor_path(w) and w.group * w.window <= 64 and 5 * ctas >= tiles
+
+
 def launches_per_call(w) -> int:
     """Kernels one ecokv_evict call launches: the persistent tensor-core
     streaming kernel (once per window-row group) or the two CUDA-core passes,
     then the finalize/select kernel (one thread-block cluster per head, or one
-    CTA per head past 131072 candidates) and the compaction kernel."""
+    CTA per head past 131072 candidates) and the compaction kernel; for a few
+    short heads one kernel in place of the streaming and finalize kernels."""
+    if short_units(w):
+        return 2
     return (row_groups(w) if tensor_path(w) else 2) + 2
 
 

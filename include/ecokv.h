@@ -43,8 +43,11 @@
  *  - Paths: bf16 inputs with n >= 128 stream K through a persistent
  *    tensor-core kernel, one launch for both of its passes over K, or one
  *    launch per group of at most 120 window rows when (h_q / h_kv) * window
- *    exceeds 120 (each group reads K twice); fp32 inputs, shorter caches and
- *    ECOKV_FLAG_FORCE_SIMT take the CUDA-core passes.  Every path is
+ *    exceeds 120 (each group reads K twice); a few short heads (up to 5120
+ *    keys and 64 window rows, one cluster of CTAs per head on the device at
+ *    once, no variant flag but the centroid's and the MixKV sign, the default
+ *    schedule) take one kernel that also scores and selects; fp32 inputs,
+ *    shorter caches and ECOKV_FLAG_FORCE_SIMT take the CUDA-core passes.  Every path is
  *    deterministic; scores may differ in their last bits between paths and
  *    between streaming schedules (ecokv_params.sched_*), within the
  *    documented tolerances.
@@ -294,7 +297,8 @@ ecokv_status ecokv_device_status(void* ws, void* stream);
  * events[0] before the streaming kernel(s), events[1] after them, events[2]
  * after the finalize / select kernel and (ecokv_evict only) events[3] after
  * the compaction kernel, so that cudaEventElapsedTime gives each stage's
- * device time.  Returns ECOKV_ERR_INVALID_ARG if events != NULL and n != 4. */
+ * device time (a few short heads: one kernel does the first two stages, and
+ * events[2] follows events[1] directly).  Returns ECOKV_ERR_INVALID_ARG if events != NULL and n != 4. */
 ecokv_status ecokv_set_stage_events(void* const* events, int n);
 
 /* Static text for a status code. */

@@ -2,9 +2,11 @@
 // launches.  Every entry point validates on the host and returns before
 // launching anything when an argument is wrong.
 //
-// Paths.  bf16 inputs with n >= 128 stream K through the persistent
-// tensor-core kernel (tc_pass.cu, one launch for both passes, or one launch
-// per group of at most 120 window rows when (h_q/h_kv)*W exceeds 120);
+// Paths.  A few short bf16 heads take one cluster per head for the passes, the
+// scores and the selection together (tc_short.cu, one launch); other bf16
+// inputs with n >= 128 stream K through the persistent tensor-core kernel
+// (tc_pass.cu, one launch for both passes, or one launch per group of at most
+// 120 window rows when (h_q/h_kv)*W exceeds 120);
 // fp32 inputs, other shapes and calls with ECOKV_FLAG_FORCE_SIMT use the
 // CUDA-core passes (score_simt.cu, two launches).  Either way one more launch
 // (finalize_select.cu) turns the pass-2 outputs into scores, selects and
@@ -267,6 +269,45 @@ static ecokv_status run_tc_group(const ecokv_params& p, const Layout& L, const v
   return ECOKV_OK;
 }
 
+// Short units: score (and, with f.idx, select) by one cluster per unit in one
+// launch.  CTAs a unit takes, 0 where the call goes another way: the variants
+// that need another launch between the passes and the finalisation, a streaming
+// schedule asked for, and the injected stall, which lives in the persistent
+// kernel.
+static int short_ctas(const ecokv_params& p, ecokv_dtype dt) {
+  if (!use_tensor_path(p, dt) || p.sched_wave != 0 || p.sched_lag != 0) return 0;
+  if (p.flags & (ECOKV_FLAG_VNORM_IMP | ECOKV_FLAG_WINSOR_1 | ECOKV_FLAG_WINSOR_5 | ECOKV_FLAG_MAD | ECOKV_FLAG_TEST_STALL))
+    return 0;
+  return short_cluster((p.h_q / p.h_kv) * p.window, (p.n + 127) / 128, (long long)p.n_layers * p.h_kv, num_sms());
+}
+static ecokv_status run_short(const ecokv_params& p, const Layout& L, const void* K, const void* Q, char* ws,
+                              const FinalArgs& f, int C, cudaStream_t s) {
+  ShortArgs a{};
+  a.U = L.U;
+  a.N = p.n;
+  a.W = p.window;
+  a.R = L.R;
+  a.g = p.h_q / p.h_kv;
+  a.h_kv = p.h_kv;
+  a.h_q = p.h_q;
+  a.Tv = L.Tv;
+  a.T = (p.n + 127) / 128;
+  a.kbar_n = kbar_count(p, L);
+  a.q_rows = p.n_layers * p.h_q * p.window;
+  a.ustat_stride = L.ustat_stride;
+  a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)p.d));
+  a.timeout_ns = wait_limit_ns(p);
+  a.Q = Q;
+  a.K = K;
+  a.ustat = reinterpret_cast<float*>(ws + L.ustat);
+  a.p2part = reinterpret_cast<float*>(ws + L.p2part);
+  a.simp = reinterpret_cast<float*>(ws + L.simp);
+  a.dE = reinterpret_cast<float*>(ws + L.dE);
+  a.cosv = reinterpret_cast<float*>(ws + L.cosv);
+  a.status = reinterpret_cast<unsigned*>(ws + L.status);
+  return launch_short(a, f, C, s) == cudaSuccess ? ECOKV_OK : ECOKV_ERR_CUDA;
+}
+
 // CUDA-core streaming passes: fill the per-token arrays and unit statistics.
 static ecokv_status run_simt_passes(const ecokv_params& p, ecokv_dtype dt, const void* K, const void* Q, char* ws,
                                     cudaStream_t s) {
@@ -404,11 +445,16 @@ ecokv_status ecokv_score(const ecokv_params* p, ecokv_dtype dtype, const void* K
   f.dbg = dbg;
   if ((st = robust_check(*p, L)) != ECOKV_OK) return st;
   stage_event(0, s);
-  st = tc ? run_tc_passes(*p, K, Qwin, w, s) : run_simt_passes(*p, dtype, K, Qwin, w, s);
-  if (st != ECOKV_OK) return st;
-  stage_event(1, s);
-  if ((st = robust_launch(*p, L, w, f, s)) != ECOKV_OK) return st;
-  if (run_finalize(f, L.U, false, s) != ECOKV_OK) return ECOKV_ERR_CUDA;
+  if (const int C = short_ctas(*p, dtype)) {
+    if ((st = run_short(*p, L, K, Qwin, w, f, C, s)) != ECOKV_OK) return st;
+    stage_event(1, s);
+  } else {
+    st = tc ? run_tc_passes(*p, K, Qwin, w, s) : run_simt_passes(*p, dtype, K, Qwin, w, s);
+    if (st != ECOKV_OK) return st;
+    stage_event(1, s);
+    if ((st = robust_launch(*p, L, w, f, s)) != ECOKV_OK) return st;
+    if (run_finalize(f, L.U, false, s) != ECOKV_OK) return ECOKV_ERR_CUDA;
+  }
   stage_event(2, s);
   return ECOKV_OK;
 }
@@ -472,12 +518,17 @@ ecokv_status ecokv_evict_adaptive(const ecokv_params* p, ecokv_dtype dtype, cons
   f.lambda = lambda;
   if ((st = vnorm_check(*p, L)) != ECOKV_OK || (st = robust_check(*p, L)) != ECOKV_OK) return st;
   stage_event(0, s);
-  st = tc ? run_tc_passes(*p, K, Qwin, w, s) : run_simt_passes(*p, dtype, K, Qwin, w, s);
-  if (st != ECOKV_OK) return st;
-  if ((st = vnorm_launch(*p, dtype, L, V, w, f, s)) != ECOKV_OK) return st;
-  if ((st = robust_launch(*p, L, w, f, s)) != ECOKV_OK) return st;
-  stage_event(1, s);
-  if (run_finalize(f, L.U, false, s) != ECOKV_OK) return ECOKV_ERR_CUDA;
+  if (const int C = short_ctas(*p, dtype)) {
+    if ((st = run_short(*p, L, K, Qwin, w, f, C, s)) != ECOKV_OK) return st;
+    stage_event(1, s);
+  } else {
+    st = tc ? run_tc_passes(*p, K, Qwin, w, s) : run_simt_passes(*p, dtype, K, Qwin, w, s);
+    if (st != ECOKV_OK) return st;
+    if ((st = vnorm_launch(*p, dtype, L, V, w, f, s)) != ECOKV_OK) return st;
+    if ((st = robust_launch(*p, L, w, f, s)) != ECOKV_OK) return st;
+    stage_event(1, s);
+    if (run_finalize(f, L.U, false, s) != ECOKV_OK) return ECOKV_ERR_CUDA;
+  }
   // 2. one top-h_kv (B - W) per layer over its heads' concatenated scores
   //    ([h_kv][Tv] per layer is contiguous), ties to the lower (head, position)
   AdaptArgs a{};
@@ -541,12 +592,17 @@ static ecokv_status evict_impl(const ecokv_params* p, ecokv_dtype dtype, const v
   }
   if ((st = vnorm_check(*p, L)) != ECOKV_OK || (st = robust_check(*p, L)) != ECOKV_OK) return st;
   stage_event(0, s);
-  st = tc ? run_tc_passes(*p, K, Qwin, w, s) : run_simt_passes(*p, dtype, K, Qwin, w, s);
-  if (st != ECOKV_OK) return st;
-  if ((st = vnorm_launch(*p, dtype, L, V, w, f, s)) != ECOKV_OK) return st;
-  if ((st = robust_launch(*p, L, w, f, s)) != ECOKV_OK) return st;
-  stage_event(1, s);
-  if (run_finalize(f, L.U, true, s) != ECOKV_OK) return ECOKV_ERR_CUDA;
+  if (const int C = short_ctas(*p, dtype)) {
+    if ((st = run_short(*p, L, K, Qwin, w, f, C, s)) != ECOKV_OK) return st;
+    stage_event(1, s);
+  } else {
+    st = tc ? run_tc_passes(*p, K, Qwin, w, s) : run_simt_passes(*p, dtype, K, Qwin, w, s);
+    if (st != ECOKV_OK) return st;
+    if ((st = vnorm_launch(*p, dtype, L, V, w, f, s)) != ECOKV_OK) return st;
+    if ((st = robust_launch(*p, L, w, f, s)) != ECOKV_OK) return st;
+    stage_event(1, s);
+    if (run_finalize(f, L.U, true, s) != ECOKV_OK) return ECOKV_ERR_CUDA;
+  }
   stage_event(2, s);
   if (launch_compact(c, dtype, L.U, s) != cudaSuccess) return ECOKV_ERR_CUDA;
   stage_event(3, s);

@@ -71,15 +71,14 @@
 #include "finalize_select.cuh"
 #include "ptx.cuh"
 #include "tc_pass.cuh"
+#include "tc_tile.cuh"
 
 namespace ecokv {
 namespace {
 
 using namespace ptx;
 
-constexpr int kTile = 128;
 constexpr int kCtl = 256;              // threads before the tile groups: control warps 0..3, stats warps 4..7
-constexpr uint32_t kTileBytes = kTile * kD * 2;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSigmaCol = 448;    // sum accumulators, 16 columns for each item slot
 constexpr int kStatRows = 5;           // kbar in three terms, mu in two
@@ -155,12 +154,6 @@ static_assert(smem_ok<8>() && smem_ok<16>() && smem_ok<32>() && smem_ok<56>() &&
 
 __device__ __forceinline__ unsigned* abort_flag(const TcArgs& a) { return a.sync + 1; }
 __device__ __forceinline__ unsigned* arrivals(const TcArgs& a, int u) { return a.sync + 4 + u; }
-
-__device__ __forceinline__ unsigned long long now_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
 
 __device__ void raise_abort(const TcArgs& a, unsigned code, unsigned detail) {
   if (atomicCAS(a.status, 0u, code) == 0u) a.status[1] = detail;
@@ -246,15 +239,6 @@ __device__ bool wait_count(const unsigned* f, unsigned target, const TcArgs& a, 
   return true;
 }
 
-__device__ __forceinline__ uint32_t sw128(int row, int chunk16) {
-  return (uint32_t)(row * 128 + ((chunk16 ^ (row & 7)) << 4));
-}
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
-
 // Pass-2 rows of the B operand (128-byte-swizzled, K-major): rows RP..RP+2
 // hold kbar split into three bf16 terms (hi, mid, lo), rows RP+3, RP+4 hold
 // mu_hi and mu_lo, all from the unit statistics copy; the window queries in
@@ -277,120 +261,6 @@ __device__ __forceinline__ void build_stat_rows(uint8_t* qb, const float* ust, i
   const uint4 val = make_uint4(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]), pack_bf16x2(o[4], o[5]),
                                pack_bf16x2(o[6], o[7]));
   *reinterpret_cast<uint4*>(qb + (j >> 3) * (Cfg<RP>::kNP * 128) + sw128(RP + which, j & 7)) = val;
-}
-
-// Joint (max, sum) of partial softmax sums: (m1, z1) + (m2, z2) with z
-// relative to 2^m; an empty pair has m = -inf, z = 0.
-__device__ __forceinline__ void combine_maxsum(float& m, float& z, float m2, float z2) {
-  const float M = fmaxf(m, m2);
-  const float Ms = M == -INFINITY ? 0.f : M;
-  z = z * ex2(m - Ms) + z2 * ex2(m2 - Ms);
-  m = M;
-}
-
-// Sum of v[j] over the lanes of a warp for every j < N, scattered: five
-// halving steps leave lane l with the rows base .. base + kOut - 1 below lim.
-template <int N>
-struct ScatterSum {
-  static constexpr int kH1 = (N + 1) / 2, kH2 = (kH1 + 1) / 2, kH3 = (kH2 + 1) / 2, kH4 = (kH3 + 1) / 2;
-  static constexpr int kOut = (kH4 + 1) / 2;
-  template <int n>
-  __device__ __forceinline__ static void step(float (&v)[N], int o, int lane, int& base, int& lim) {
-    constexpr int h = (n + 1) / 2;
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int j = 0; j < h; ++j) {
-      const float hi = j + h < n ? v[j + h] : 0.f;
-      const float keep = up ? hi : v[j], send = up ? v[j] : hi;
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-    if (up) base += h;
-    else lim = min(lim, base + h);
-  }
-  __device__ __forceinline__ static void run(float (&v)[N], int lane, int& base, int& lim) {
-    base = 0;
-    lim = N;
-    step<N>(v, 16, lane, base, lim);
-    step<kH1>(v, 8, lane, base, lim);
-    step<kH2>(v, 4, lane, base, lim);
-    step<kH3>(v, 2, lane, base, lim);
-    step<kH4>(v, 1, lane, base, lim);
-  }
-};
-
-// One pass-1 tile of a warp: the partial softmax sums of its rows, one key a
-// lane.  z[c] += 2^(x - m) with m a reference per row that the warp's lanes
-// share: the logit of the first key of the warp's first tile of the item
-// (where that key is not visible to the row none of the warp's keys is; 0
-// then), kept negated in shared memory and raised in the rare tile that
-// exceeds it by more than 2^6.  Rows past R run along, their sums are not
-// kept.  vis_from: a row with window position j sees the lane's key iff j >=
-// vis_from (INT_MAX for a key past N); j0: the first row's window position.
-// The columns are read kCW at a time: a read costs about 0.25 us whatever its
-// width (in eights, 56 rows took 2.3 us a tile).
-template <int RP>
-__device__ __forceinline__ void pass1_rows(uint32_t taddr, float (&z)[RP], float* ref, float scale, bool first,
-                                           bool all_vis, int vis_from, int j0, int W, int lane, uint64_t* bar_empty) {
-  constexpr int kCW = Cfg<RP>::kCW;
-  int jw = j0;
-#pragma unroll
-  for (int c0 = 0; c0 < RP; c0 += kCW) {
-    uint32_t rc[kCW];
-    tmem_ld<kCW>(taddr + (uint32_t)c0, rc);
-    tmem_wait_ld();
-    if (c0 + kCW == RP) {
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_empty);
-    }
-    if (first) {
-      if (lane == 0) {
-        int jf = jw;
-#pragma unroll
-        for (int c = 0; c < kCW; ++c) {
-          const bool vis = all_vis || jf >= vis_from;
-          if (++jf == W) jf = 0;
-          ref[c0 + c] = vis ? -(__uint_as_float(rc[c]) * scale) : 0.f;
-        }
-      }
-      __syncwarp();
-    }
-    {
-      float mx = -INFINITY;
-#pragma unroll
-      for (int c = 0; c < kCW; c += 4) {
-        const float4 nr = *reinterpret_cast<const float4*>(ref + c0 + c);
-        rc[c] = __float_as_uint(fmaf(__uint_as_float(rc[c]), scale, nr.x));
-        rc[c + 1] = __float_as_uint(fmaf(__uint_as_float(rc[c + 1]), scale, nr.y));
-        rc[c + 2] = __float_as_uint(fmaf(__uint_as_float(rc[c + 2]), scale, nr.z));
-        rc[c + 3] = __float_as_uint(fmaf(__uint_as_float(rc[c + 3]), scale, nr.w));
-      }
-      if (!all_vis) {
-#pragma unroll
-        for (int c = 0; c < kCW; ++c) {
-          if (!(jw >= vis_from)) rc[c] = 0xff800000u;  // -inf
-          if (++jw == W) jw = 0;
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < kCW; ++c) mx = fmaxf(mx, __uint_as_float(rc[c]));
-      if (__any_sync(0xffffffffu, mx > 64.f)) {
-#pragma unroll
-        for (int c = 0; c < kCW; ++c) {
-          const float d = __uint_as_float(rc[c]);
-          const float up = redux_max(d);
-          if (up > 20.f) {
-            z[c0 + c] *= ex2(-up);
-            rc[c] = __float_as_uint(d - up);
-            if (lane == 0) ref[c0 + c] -= up;
-          }
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < kCW; ++c) z[c0 + c] += ex2(__uint_as_float(rc[c]));
-    }
-  }
-  __syncwarp();
 }
 
 template <int RP>
@@ -469,25 +339,6 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
 
     // first tile of an item that is this group's (tile counter mod kGroups)
     auto first_own = [&](uint32_t tc0) { return ((uint32_t)grp + kGroups - tc0 % kGroups) % kGroups; };
-    // squared norm of this thread's key in a stage (packed fp32 pairs), the
-    // same arithmetic in both passes
-    auto norm2 = [&](uint32_t stage) -> float {
-      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int hb = 0; hb < 2; ++hb) {
-        const uint8_t* row = s.ktile[stage] + hb * (kTileBytes / 2) + kk * 128;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const uint4 v = *reinterpret_cast<const uint4*>(row + ((c ^ (kk & 7)) << 4));
-          sq_acc_bf16x2(v.x, acc[0], acc[1]);
-          sq_acc_bf16x2(v.y, acc[2], acc[3]);
-          sq_acc_bf16x2(v.z, acc[4], acc[5]);
-          sq_acc_bf16x2(v.w, acc[6], acc[7]);
-        }
-      }
-      return ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
-    };
-
     for (uint32_t seq = 0; ok; ++seq) {
       const uint32_t slot = seq % kIQ, qphase = (seq / kIQ) & 1u;
       if (!(ok = wait_warp(&s.item_full[slot], qphase, a, 10u))) break;
@@ -513,22 +364,10 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
           const bool valid = i < a.N;
           if (!(ok = wait_warp(&s.full[stage], sph, a, 22u))) break;
           if (sums) {
-            const float n2 = norm2(stage);
+            const float n2 = key_norm2(s.ktile[stage], kk);
             __syncwarp();
             if (lane == 0) mbar_arrive(&s.empty[stage]);  // done with the key tile
-            // the sum weights w = 1/||k|| in three bf16 terms
-            const float w = valid ? rsqrtf(fmaxf(n2, 1e-24f)) : 0.f;
-            const __nv_bfloat16 whi = __float2bfloat16_rn(w);
-            const float r1 = w - __bfloat162float(whi);
-            const __nv_bfloat16 wmid = __float2bfloat16_rn(r1);
-            const __nv_bfloat16 wlo = __float2bfloat16_rn(r1 - __bfloat162float(wmid));
-            uint8_t* base = s.wbuf[stage][kk >> 6] + (kk & 7) * 2;
-            const int j = (kk & 63) >> 3;
-            if (a.kbar_n < a.N)  // non-window centroid: the window keys leave the sum of k
-              *reinterpret_cast<__nv_bfloat16*>(base + sw128(0, j)) = __float2bfloat16_rn(i < a.kbar_n ? 1.f : 0.f);
-            *reinterpret_cast<__nv_bfloat16*>(base + sw128(1, j)) = whi;
-            *reinterpret_cast<__nv_bfloat16*>(base + sw128(2, j)) = wmid;
-            *reinterpret_cast<__nv_bfloat16*>(base + sw128(3, j)) = wlo;
+            put_weights(s.wbuf[stage][0], kk, n2, valid, a.kbar_n < a.N, i < a.kbar_n);
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&s.wready[stage]);
@@ -539,7 +378,7 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
           tc_fence_after();
           const bool all_vis = it0 + kTile - 1 <= a.N - a.W;  // every window row sees every key of the tile
           const int vis_from = valid ? i - (a.N - a.W) : 0x7fffffff;
-          pass1_rows<RP>(tl + b * (uint32_t)kNP, z, ref, a.scale_log2, first, all_vis, vis_from, j0, a.W, lane,
+          pass1_rows<RP, C::kCW>(tl + b * (uint32_t)kNP, z, ref, a.scale_log2, first, all_vis, vis_from, j0, a.W, lane,
                          &s.tmem_empty[b]);
           first = false;
         }
@@ -585,7 +424,7 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
           const int i = i0 + (int)(ntiles - 1u - t) * kTile + kk;  // pass 2 walks the item backwards
           const bool valid = i < a.N;
           if (!(ok = wait_warp(&s.full[stage], sph, a, 23u))) break;
-          const float n2 = sums ? norm2(stage) : 0.f;
+          const float n2 = sums ? key_norm2(s.ktile[stage], kk) : 0.f;
           __syncwarp();
           if (lane == 0) mbar_arrive(&s.empty[stage]);
           if (!(ok = wait_warp(&s.tmem_full[b], tph, a, 14u))) break;
@@ -622,22 +461,7 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
             const float kmu = __uint_as_float(st[3]) + __uint_as_float(st[4]);
             float d2 = fmaf(-2.f, kkb, n2) + ksq;
             if (valid && d2 < 0.015625f * (n2 + ksq)) {
-              // cancellation regime: recompute |k - kbar|^2 from the key row
-              const uint4* row = reinterpret_cast<const uint4*>(a.K) + ((size_t)u * a.N + i) * 16;
-              float dp[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-              for (int c = 0; c < 16; ++c) {
-                const uint4 kv = __ldg(row + c);
-                const uint32_t w4[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-                for (int t2 = 0; t2 < 4; ++t2) {
-                  const float dl = __uint_as_float(w4[t2] << 16) - kbv[c * 8 + 2 * t2];
-                  const float dh = __uint_as_float(w4[t2] & 0xffff0000u) - kbv[c * 8 + 2 * t2 + 1];
-                  dp[t2] = fmaf(dl, dl, dp[t2]);
-                  dp[t2] = fmaf(dh, dh, dp[t2]);
-                }
-              }
-              d2 = (dp[0] + dp[1]) + (dp[2] + dp[3]);
+              d2 = direct_d2(reinterpret_cast<const uint4*>(a.K) + ((size_t)u * a.N + i) * 16, kbv);
             }
             const float dEv = sqrtf(fmaxf(d2, 0.f));
             const float cs = kmu * rsqrtf(fmaxf(n2, 1e-24f));
@@ -1136,6 +960,30 @@ int tc_rows(int R) {
   return 0;
 }
 
+cudaError_t tc_tensor_maps(const void* K, int N, int U, const void* Q, int q_rows, int RP, CUtensorMap* tm,
+                           CUtensorMap* tq) {
+  EncodeTiledFn enc = encode_fn();
+  if (enc == nullptr) return cudaErrorNotSupported;
+  const cuuint64_t dims[3] = {(cuuint64_t)kD, (cuuint64_t)N, (cuuint64_t)U};
+  const cuuint64_t strides[2] = {(cuuint64_t)kD * 2, (cuuint64_t)N * kD * 2};
+  const cuuint32_t box[3] = {64, (cuuint32_t)kTile, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  if (enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(K), dims, strides, box, estr,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  // window queries as a 2-D [L * h_q * W rows, 128] bf16 tensor, boxes of
+  // [RP rows x 64 columns] with the same 128-byte swizzle as the key tiles
+  const cuuint64_t qdims[2] = {(cuuint64_t)kD, (cuuint64_t)q_rows};
+  const cuuint64_t qstrides[1] = {(cuuint64_t)kD * 2};
+  const cuuint32_t qbox[2] = {64, (cuuint32_t)RP};
+  if (enc(tq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(Q), qdims, qstrides, qbox, estr,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  return cudaSuccess;
+}
+
 cudaError_t launch_tc(const void* K, const TcArgs& args, cudaStream_t st) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1147,27 +995,9 @@ cudaError_t launch_tc(const void* K, const TcArgs& args, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     g_num_sms[dev].store(n);
   }
-  EncodeTiledFn enc = encode_fn();
-  if (enc == nullptr) return cudaErrorNotSupported;
-  CUtensorMap tm;
-  const cuuint64_t dims[3] = {(cuuint64_t)kD, (cuuint64_t)args.N, (cuuint64_t)args.U};
-  const cuuint64_t strides[2] = {(cuuint64_t)kD * 2, (cuuint64_t)args.N * kD * 2};
-  const cuuint32_t box[3] = {64, (cuuint32_t)kTile, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  if (enc(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(K), dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
-  // window queries as a 2-D [L * h_q * W rows, 128] bf16 tensor, boxes of
-  // [RP rows x 64 columns] with the same 128-byte swizzle as the key tiles
-  CUtensorMap tq;
-  const cuuint64_t qdims[2] = {(cuuint64_t)kD, (cuuint64_t)args.q_rows};
-  const cuuint64_t qstrides[1] = {(cuuint64_t)kD * 2};
-  const cuuint32_t qbox[2] = {64, (cuuint32_t)args.RP};
-  if (enc(&tq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(args.Q), qdims, qstrides, qbox, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
+  CUtensorMap tm, tq;
+  e = tc_tensor_maps(K, args.N, args.U, args.Q, args.q_rows, args.RP, &tm, &tq);
+  if (e != cudaSuccess) return e;
   switch (args.RP) {
     case 8: return launch_rp<8>(tm, tq, args, dev, st);
     case 16: return launch_rp<16>(tm, tq, args, dev, st);

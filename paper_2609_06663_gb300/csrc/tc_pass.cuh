@@ -1,6 +1,8 @@
 // Launch interface of the persistent tensor-core kernel (tc_pass.cu).
 #pragma once
 
+#include <cuda.h>
+
 #include "ecokv_internal.cuh"
 
 namespace ecokv {
@@ -42,5 +44,36 @@ int tc_rows(int R);
 // can meet.
 int tc_record_slots(int T, int L);
 cudaError_t launch_tc(const void* K, const TcArgs& args, cudaStream_t st);
+
+// Tensor maps of the keys [U][N][d] (boxes of 128 keys x 64 dimensions) and of
+// the window queries [q_rows][d] (boxes of RP rows x 64), 128-byte swizzle.
+cudaError_t tc_tensor_maps(const void* K, int N, int U, const void* Q, int q_rows, int RP, CUtensorMap* tm,
+                           CUtensorMap* tq);
+
+// Short units (tc_short.cu): the whole score, and the selection, of each unit
+// by one thread-block cluster that holds its keys in shared memory.
+constexpr int kShortTiles = 5;    // key tiles a CTA holds
+constexpr int kShortCtas = 8;     // CTAs a unit may take
+struct ShortArgs {
+  int U, N, W, R, g, h_kv, h_q, Tv, T;
+  int kbar_n;                       // keys 0 .. kbar_n - 1 form the centroid
+  int q_rows;                       // rows of the window-query tensor
+  int ustat_stride;
+  float scale_log2;
+  unsigned long long timeout_ns;    // limit of every bounded wait (global timer)
+  const void* Q;
+  const void* K;
+  float* ustat;                     // [U][ustat_stride]: only ||mu||^2 is written
+  float* p2part;                    // [U][C][kP2Stride]
+  float* simp;
+  float* dE;
+  float* cosv;
+  unsigned* status;
+};
+// CTAs a unit takes, or 0 where this kernel does not apply: R window rows, T
+// tiles a unit, U units on a device of `sms` SMs.
+int short_cluster(int R, int T, long long U, int sms);
+// f: the finalisation's arguments (f.nchunks is set here); scores only when f.idx is null.
+cudaError_t launch_short(const ShortArgs& a, FinalArgs f, int C, cudaStream_t st);
 
 }  // namespace ecokv
