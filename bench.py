@@ -103,10 +103,11 @@ SMS = 152  # of a GB300
 
 def short_units(w) -> bool:
     """Few short heads take one launch for both passes, scores and selection:
-    up to 40 tiles of 128 keys and 64 window rows, one cluster per head, all
-    clusters (at most five tiles a CTA) on the GPU at once."""
+    up to 64 window rows, one cluster per head, all clusters (at most five
+    tiles of 128 keys a CTA, eight CTAs or, for up to seven heads, sixteen) on
+    the GPU at once."""
     tiles = (w.n + 127) // 128
-    ctas = min(8, tiles, SMS // w.units)
+    ctas = min(16 if tiles > 16 and w.units <= 7 else 8, tiles, SMS // w.units)
     return tensor_path(w) and w.group * w.window <= 64 and 5 * ctas >= tiles
 
 

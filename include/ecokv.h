@@ -43,9 +43,10 @@
  *  - Paths: bf16 inputs with n >= 128 stream K through a persistent
  *    tensor-core kernel, one launch for both of its passes over K, or one
  *    launch per group of at most 120 window rows when (h_q / h_kv) * window
- *    exceeds 120 (each group reads K twice); a few short heads (up to 5120
- *    keys and 64 window rows, one cluster of CTAs per head on the device at
- *    once, no variant flag but the centroid's and the MixKV sign, the default
+ *    exceeds 120 (each group reads K twice); a few short heads (up to 64
+ *    window rows, one cluster of CTAs per head holding all its keys, every
+ *    head's on the device at once: up to 10240 keys for 7 heads, 5120 for 19,
+ *    640 for 152; no variant flag but the centroid's and the MixKV sign, the default
  *    schedule) take one kernel that also scores and selects; fp32 inputs,
  *    shorter caches and ECOKV_FLAG_FORCE_SIMT take the CUDA-core passes.  Every path is
  *    deterministic; scores may differ in their last bits between paths and

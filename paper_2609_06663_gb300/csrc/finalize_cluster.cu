@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(kCThreads, Shape<kSh>::kMinCtas) finalize_clus
 }
 
 template <int kSh>
-cudaError_t set_attrs() {
+cudaError_t set_attrs(bool nonportable) {
   const int bytes = (int)sizeof(ClusterSmem<kSh>);
   const void* kernels[5] = {(const void*)finalize_cluster_kernel<0, kSh, false>,
                             (const void*)finalize_cluster_kernel<1, kSh, false>,
@@ -35,8 +35,7 @@ cudaError_t set_attrs() {
                             (const void*)finalize_cluster_kernel<2, kSh, false>};
   for (const void* k : kernels) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && Shape<kSh>::kMaxCluster > 8)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess && nonportable) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -70,15 +69,21 @@ cudaError_t launch_shape(const FinalArgs& f, int U, int C, bool select_only, cud
 // Per device: the attributes set, and whether clusters of 16 CTAs of the
 // longest shape can be resident (cudaOccupancyMaxActiveClusters > 0).
 std::atomic<int> g_setup[64];  // 0 = not yet, 1 = set, clusters of 16 unavailable, 2 = set and available
+std::atomic<int> g_sms[64];    // SMs, set before g_setup
 
 int device_setup() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
   int st = g_setup[dev].load();
   if (st != 0) return st;
-  if (set_attrs<0>() != cudaSuccess || set_attrs<1>() != cudaSuccess || set_attrs<2>() != cudaSuccess) return -1;
+  if (set_attrs<0>(false) != cudaSuccess || set_attrs<1>(false) != cudaSuccess || set_attrs<2>(false) != cudaSuccess ||
+      set_attrs<3>(false) != cudaSuccess)
+    return -1;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return -1;
+  g_sms[dev].store(sms);
   st = 1;
-  if (set_attrs<3>() == cudaSuccess) {
+  if (set_attrs<0>(true) == cudaSuccess && set_attrs<3>(true) == cudaSuccess) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(16u * 16u, 1, 1);
     cfg.blockDim = dim3(kCThreads, 1, 1);
@@ -100,19 +105,32 @@ int device_setup() {
   return st;
 }
 
-// Shape and cluster size for units of Tv candidates: the shortest shape whose
-// cluster takes them; shape -1 when none does.
-void pick_shape(int Tv, int long_ok, int& sh, int& C) {
+// Shape and cluster size for U units of Tv candidates; shape -1 when none takes
+// them.  The fewest candidates a thread whose CTAs are all resident at once;
+// failing that (many units) the fewest in clusters of at most four.  One layer
+// of 4 heads x 32768 keys: 16 CTAs of 8 a thread 15 us, 4 of 32 a thread 25 us;
+// 28 layers x 4 heads of that length: 3 waves of the former, one of the latter.
+void pick_shape(int Tv, long long U, int long_ok, int sms, int& sh, int& C) {
   const int t = Tv > 0 ? Tv : 1;
   const int cap[4] = {Shape<0>::kCap, Shape<1>::kCap, Shape<2>::kCap, Shape<3>::kCap};
-  const int most[4] = {Shape<0>::kMaxCluster, Shape<1>::kMaxCluster, Shape<2>::kMaxCluster,
+  const int most[4] = {long_ok ? Shape<0>::kMaxCluster : 8, Shape<1>::kMaxCluster, Shape<2>::kMaxCluster,
                        long_ok ? Shape<3>::kMaxCluster : 8};
+  const int resident[4] = {Shape<0>::kMinCtas, Shape<1>::kMinCtas, Shape<2>::kMinCtas, Shape<3>::kMinCtas};
   for (sh = 0; sh < 4; ++sh) {
     C = (t + cap[sh] - 1) / cap[sh];
-    if (C <= most[sh]) return;
+    if (C <= most[sh] && U * C <= (long long)resident[sh] * sms) return;
+  }
+  for (sh = 0; sh < 4; ++sh) {
+    C = (t + cap[sh] - 1) / cap[sh];
+    if (C <= (sh < 3 ? 4 : most[3])) return;
   }
   sh = -1;
   C = 0;
+}
+
+int current_sms() {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_sms[dev].load() : 0;
 }
 
 }  // namespace
@@ -121,7 +139,7 @@ bool cluster_finalize_fits(int Tv) {
   const int st = device_setup();
   if (st < 0) return false;
   int sh, C;
-  pick_shape(Tv, st == 2, sh, C);
+  pick_shape(Tv, 1, st == 2, current_sms(), sh, C);
   return sh >= 0;
 }
 
@@ -129,7 +147,7 @@ cudaError_t launch_finalize_cluster(const FinalArgs& f, int U, bool select_only,
   const int st = device_setup();
   if (st < 0) return cudaErrorUnknown;
   int sh, C;
-  pick_shape(f.Tv, st == 2, sh, C);
+  pick_shape(f.Tv, U, st == 2, current_sms(), sh, C);
   switch (sh) {
     case 0: return launch_shape<0>(f, U, C, select_only, s);
     case 1: return launch_shape<1>(f, U, C, select_only, s);

@@ -3,12 +3,12 @@
 // (finalize_select.cuh), spread over the cluster so that every SM takes part,
 // with the cluster-wide reductions done through distributed shared memory.
 //
-// Shapes: 8, 16 or 32 candidates a thread and up to 4 CTAs (units of up to
-// 8192, 16384 and 32768 candidates), or 32 a thread and up to 16 CTAs (up to
-// 131072).  Four CTAs a unit at the most where that is enough: at three or
-// more CTAs per SM the 112 units of a prefill (28 layers x 4 KV heads) are
-// then resident in one wave (clusters of 8 would need one and a half), and the
-// kernel, all latency, takes one unit's time.
+// Shapes: 8, 16 or 32 candidates a thread and up to 16, 4 or 4 CTAs, or 32 a
+// thread and up to 16 CTAs (units of up to 131072 candidates).  The kernel is
+// all latency, and shorter the less a thread has to do, so a unit is spread as
+// widely as leaves every unit's CTAs resident at once (three or four per SM):
+// four heads of 32760 candidates on 16 CTAs each, the 112 units of a prefill
+// (28 layers x 4 KV heads) of that length on four each.
 //
 // CTA rank r of the cluster owns candidates [r * cap, (r + 1) * cap) of the
 // unit (cap = 256 threads x kJ); thread t of it owns the kJ consecutive
@@ -65,7 +65,7 @@ template <int kSh>
 struct Shape {
   static constexpr int kJ = kSh == 4 ? 4 : (kSh == 0 ? 8 : (kSh == 1 ? 16 : 32));  // candidates a thread owns
   static constexpr int kCap = kCThreads * kJ;                     // candidates a CTA owns
-  static constexpr int kMaxCluster = kSh == 3 ? 16 : (kSh == 4 ? 8 : 4);           // CTAs a unit may take
+  static constexpr int kMaxCluster = kSh == 1 || kSh == 2 ? 4 : 16;              // CTAs a unit may take
   static constexpr int kQ = kCap + 2 * kHalo;                     // staged raw votes
   static constexpr int kBins = kSh == 1 || kSh == 2 ? 2048 : 1024;
   static constexpr int kMinCtas = kSh == 1 ? 3 : 4;               // resident CTAs per SM asked of the compiler
@@ -452,10 +452,14 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
         el += __fadd_rn(__fsub_rn(eh, __fsub_rn(t, b)), __fsub_rn(q, b)) + fmaf(x, c, -q);
         eh = t;
       };
-      // sm.edge[l] = raw[l] for l < h, raw[Tv - 2h + l] for h <= l < 2h
-      for (int j = 0; j < Tv && j < h; ++j) add(pool_smem ? sm.edge[j] : ld(raw + j), h - j);
-      for (int j = (Tv - h > 0 ? Tv - h : 0); j < Tv; ++j)
-        add(pool_smem ? sm.edge[j - Tv + 2 * h] : ld(raw + j), h - (Tv - 1 - j));
+      if (pool_smem) {
+        // sm.edge[l] = raw[l] for l < h, raw[Tv - 2h + l] for h <= l < 2h
+        for (int j = 0; j < Tv && j < h; ++j) add(sm.edge[j], h - j);
+        for (int j = (Tv - h > 0 ? Tv - h : 0); j < Tv; ++j) add(sm.edge[j - Tv + 2 * h], h - (Tv - 1 - j));
+      } else {
+        for (int j = 0; j < Tv && j < h; ++j) add(ld(raw + j), h - j);
+        for (int j = (Tv - h > 0 ? Tv - h : 0); j < Tv; ++j) add(ld(raw + j), h - (Tv - 1 - j));
+      }
       const double edge = (double)eh + (double)el;
       sm.dsc[0] = (double)f.pool * (double)s_raw - edge;  // kp * Tv * mean(S_imp)
     } else if (tid == 96) {

@@ -53,7 +53,7 @@ cudaError_t tc_tensor_maps(const void* K, int N, int U, const void* Q, int q_row
 // Short units (tc_short.cu): the whole score, and the selection, of each unit
 // by one thread-block cluster that holds its keys in shared memory.
 constexpr int kShortTiles = 5;    // key tiles a CTA holds
-constexpr int kShortCtas = 8;     // CTAs a unit may take
+constexpr int kShortCtas = 16;    // CTAs a unit may take
 struct ShortArgs {
   int U, N, W, R, g, h_kv, h_q, Tv, T;
   int kbar_n;                       // keys 0 .. kbar_n - 1 form the centroid

@@ -1,4 +1,4 @@
-// Short units (one (layer, KV head) of up to 40 tiles of 128 keys) on the
+// Short units (one (layer, KV head) of up to 80 tiles of 128 keys) on the
 // tensor cores: both passes over the keys, the scores and the selection in one
 // launch, one thread-block cluster per unit.
 //
@@ -426,6 +426,10 @@ cudaError_t launch_short_rp(const CUtensorMap& tm, const CUtensorMap& tq, const 
     const cudaError_t e = cudaFuncSetAttribute(short_unit_kernel<RP, kSelect>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    // (clusters past 8 are asked for only where max_clusters16 has seen them allowed)
+    if (cudaFuncSetAttribute(short_unit_kernel<RP, kSelect>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+        cudaSuccess)
+      cudaGetLastError();
     g_attr_set[dev][inst].store(true);
   }
   cudaLaunchConfig_t cfg{};
@@ -445,13 +449,51 @@ cudaError_t launch_short_rp(const CUtensorMap& tm, const CUtensorMap& tq, const 
 
 }  // namespace
 
+namespace {
+// Clusters of 16 CTAs of this kernel that a device holds at once (an optional
+// size, past the portable 8): 0 = not asked yet, else the number + 1.
+std::atomic<int> g_max16[64];
+
+int max_clusters16() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int n1 = g_max16[dev].load();
+  if (n1 == 0) {
+    int n = 0;
+    const int smem = (int)sizeof(ShortSmem<64>) + 1024;  // the largest instance
+    const void* k = (const void*)short_unit_kernel<64, true>;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(16u * 16u, 1, 1);
+      cfg.blockDim = dim3(kThreads, 1, 1);
+      cfg.dynamicSmemBytes = smem;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = 16;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) n = 0;
+    }
+    cudaGetLastError();  // an unavailable configuration leaves no error behind
+    n1 = n + 1;
+    g_max16[dev].store(n1);
+  }
+  return n1 - 1;
+}
+}  // namespace
+
 int short_cluster(int R, int T, long long U, int sms) {
-  if (R > 64 || T > kShortTiles * kShortCtas) return 0;
-  // as many CTAs a unit as there are tiles, SMs and places in a cluster: the
-  // fewest tiles one after the other
+  if (R > 64 || T > kShortTiles * kShortCtas || U > sms) return 0;
+  // eight CTAs a unit (as tiles and SMs allow); past sixteen tiles sixteen
+  // CTAs where every unit's cluster of that size is resident, so that a tile
+  // group has at most two tiles up to 48 of them (4 heads x 5003 keys: 29.0
+  // against 31.0 us a call, and heads of 41 to 80 tiles need them)
   long long C = sms / U;
-  if (C > kShortCtas) C = kShortCtas;
   if (C > T) C = T;
+  if (C > 8) C = T > 16 && U <= max_clusters16() ? (C > 16 ? 16 : C) : 8;
   return C * kShortTiles >= T ? (int)C : 0;
 }
 

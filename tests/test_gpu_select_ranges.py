@@ -49,3 +49,19 @@ def test_select_at_shape_edges(t, kind):
             want = np.sort(np.lexsort((np.arange(t), -x))[:k])
             assert (idx[0, h, :k] == want).all(), f"t={t} k={k} {kind} head {h}"
             assert (idx[0, h, k:] == np.arange(t, t + window)).all()
+
+
+@pytest.mark.parametrize("t,heads", [(12000, 120), (16384, 120), (20001, 110), (32768, 114), (2048, 700), (9000, 300)])
+def test_select_many_heads(t, heads):
+    # so many heads that their CTAs take the shapes of 16 and 32 candidates a
+    # thread, or (too many for one wave in any shape) clusters of at most four
+    g = torch.Generator().manual_seed(t)
+    window, k = 4, t // 10
+    S = torch.randn(1, heads, t, generator=g)
+    S[0, ::3] = (S[0, ::3] * 8).round() / 8  # ties
+    p = E.make_params(n_layers=1, h_kv=heads, h_q=heads, n=t + window, window=window, budget=k + window)
+    idx = E.select(p, S.cuda()).cpu().numpy()
+    for h in [0, 1, 2, heads // 2, heads - 1]:
+        x = S[0, h].double().numpy()
+        want = np.sort(np.lexsort((np.arange(t), -x))[:k])
+        assert (idx[0, h, :k] == want).all(), f"t={t} head {h} of {heads}"

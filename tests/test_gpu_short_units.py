@@ -1,7 +1,7 @@
 """The short-unit kernel (one cluster per head, both passes, scores and selection
 in one launch) against the oracle, at the edges of what it takes and of how it
-splits a head: one tile to forty, one CTA a head to eight, one to five tiles a
-CTA, a ragged last tile, each instance by window rows; and against the
+splits a head: one tile to eighty, one CTA a head to sixteen, one to five tiles
+a CTA, a ragged last tile, each instance by window rows; and against the
 persistent kernel, which an explicit schedule selects."""
 import pytest
 import torch
@@ -13,11 +13,13 @@ from tests.test_gpu_parity import params_of, run_and_compare
 pytestmark = pytest.mark.gpu
 
 
-# n, heads: tiles a head and CTAs a head follow (CTAs = min(8, tiles, SMs / heads))
+# n, heads: tiles a head and CTAs a head follow (at most tiles, SMs / heads and eight,
+# or sixteen for a few heads of more than sixteen tiles)
 @pytest.mark.parametrize("n,h_kv,group,window", [
     (128, 1, 1, 1), (129, 2, 1, 8), (255, 3, 2, 8), (640, 1, 4, 4), (1024, 8, 4, 4), (1025, 8, 7, 8),
     (640, 100, 1, 8), (1280, 75, 1, 4), (1281, 50, 2, 8), (2560, 38, 1, 4), (3001, 8, 8, 8), (5003, 4, 7, 8),
-    (5120, 19, 2, 16), (5120, 1, 4, 16)], ids=lambda v: str(v))
+    (5120, 19, 2, 16), (5120, 1, 4, 16),
+    (2049, 7, 4, 8), (6000, 3, 8, 8), (8200, 7, 1, 8), (10240, 2, 7, 8)], ids=lambda v: str(v))
 def test_short_unit_shapes(n, h_kv, group, window):
     units = None if h_kv <= 8 else [(0, 0), (0, h_kv // 2), (0, h_kv - 1)]
     run_and_compare(small_workload(n, h_kv=h_kv, group=group, window=window, budget=max(window, n // 10), dtype="bf16",
