@@ -236,6 +236,9 @@ __global__ void __launch_bounds__(kThreads) pass1_kernel(ScoreArgs a) {
   float* mrow = red + kWarps * 32;                                   // [RB]
   __shared__ int s_last;
 
+  // pass 2 may be scheduled from here on: it stages its own inputs and waits
+  // for this grid's end before it reads the statistics
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   stage_queries<T>(qs, a, u, Rpad);
   const int i0 = chunk * kChunk;
   load_tile<T>(ks, static_cast<const T*>(a.K) + (size_t)u * a.N * kD, i0, a.N);
@@ -285,6 +288,7 @@ __global__ void __launch_bounds__(kThreads) pass1_kernel(ScoreArgs a) {
   const float* base = a.p1part + (size_t)u * a.nchunks * a.p1_stride;
   float* us = a.ustat + (size_t)u * a.ustat_stride;
   float sk = 0.f, skh = 0.f;
+#pragma unroll 8
   for (int c = 0; c < a.nchunks; ++c) {
     sk += __ldcg(base + (size_t)c * a.p1_stride + 2 * a.R + t);
     skh += __ldcg(base + (size_t)c * a.p1_stride + 2 * a.R + kD + t);
@@ -293,15 +297,40 @@ __global__ void __launch_bounds__(kThreads) pass1_kernel(ScoreArgs a) {
   const float kb = sk * (1.f / (float)a.kbar_n), mu = skh * inv_n;
   us[ustat_kbar() + t] = kb;
   us[ustat_mu() + t] = mu;
-  for (int row = t; row < a.R; row += kThreads) {
-    float M = -INFINITY;
-    for (int c = 0; c < a.nchunks; ++c) M = fmaxf(M, __ldcg(base + (size_t)c * a.p1_stride + row));
-    float Z = 0.f;
-    for (int c = 0; c < a.nchunks; ++c) {
-      const float m = __ldcg(base + (size_t)c * a.p1_stride + row);
-      if (m != -INFINITY) Z += __ldcg(base + (size_t)c * a.p1_stride + a.R + row) * exp2f(m - M);
+  // the rows: thread (g, row) combines the (max, sum) pairs of the chunks g, g
+  // + G, ... in order, then the G partial pairs of a row in order
+  const int G = a.R < kThreads ? min(16, kThreads / a.R) : 1;
+  for (int r0 = 0; r0 < a.R; r0 += kThreads) {
+    const int n = min(a.R - r0, kThreads), g = t / n, row = r0 + t % n;
+    float M = -INFINITY, Z = 0.f;
+    if (g < G) {
+#pragma unroll 4
+      for (int c = g; c < a.nchunks; c += G) {
+        const float m = __ldcg(base + (size_t)c * a.p1_stride + row), z = __ldcg(base + (size_t)c * a.p1_stride + a.R + row);
+        if (m != -INFINITY) {
+          const float x = fmaxf(M, m);
+          Z = Z * exp2f(M - x) + z * exp2f(m - x);
+          M = x;
+        }
+      }
     }
-    us[ustat_lse() + row] = M + log2f(Z);
+    __syncthreads();  // (qs is free: every thread is past its dot products)
+    if (g < G) {
+      qs[2 * t] = M;
+      qs[2 * t + 1] = Z;
+    }
+    __syncthreads();
+    if (t < n) {
+      for (int q = 1; q < G; ++q) {
+        const float m = qs[2 * (q * n + t)], z = qs[2 * (q * n + t) + 1];
+        if (m != -INFINITY) {
+          const float x = fmaxf(M, m);
+          Z = Z * exp2f(M - x) + z * exp2f(m - x);
+          M = x;
+        }
+      }
+      us[ustat_lse() + row] = M + log2f(Z);
+    }
   }
   const float ksq = block_sum128(kb * kb, red);
   const float msq = block_sum128(mu * mu, red);
@@ -324,12 +353,15 @@ __global__ void __launch_bounds__(kThreads) pass2_kernel(ScoreArgs a) {
   float* red = lse + Rpad;                                            // [kWarps]
 
   const float* us = a.ustat + (size_t)u * a.ustat_stride;
+  // keys and queries are the call's inputs: staged while pass 1 ends
   stage_queries<T>(qs, a, u, Rpad);
+  const int i0 = chunk * kChunk;
+  load_tile<T>(ks, static_cast<const T*>(a.K) + (size_t)u * a.N * kD, i0, a.N);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   kbar[t] = __ldcg(us + ustat_kbar() + t);
   mu[t] = __ldcg(us + ustat_mu() + t);
   for (int r = t; r < Rpad; r += kThreads) lse[r] = r < a.R ? __ldcg(us + ustat_lse() + r) : 0.f;
-  const int i0 = chunk * kChunk;
-  load_tile<T>(ks, static_cast<const T*>(a.K) + (size_t)u * a.N * kD, i0, a.N);
   __syncthreads();
 
   const int i = i0 + t;
@@ -395,8 +427,17 @@ cudaError_t launch_rb(const ScoreArgs& a, int U, cudaStream_t s) {
   pass1_kernel<T, RB><<<grid, kThreads, s1, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  pass2_kernel<T, RB><<<grid, kThreads, s2, s>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = s2;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, pass2_kernel<T, RB>, a);
 }
 
 template <typename T>
