@@ -376,6 +376,25 @@ static ecokv_status run_finalize(FinalArgs f, int U, bool do_select, cudaStream_
   return launch_finalize(f, U, do_select, s) == cudaSuccess ? ECOKV_OK : ECOKV_ERR_CUDA;
 }
 
+// The k largest of each layer's T concatenated scores, positions ascending.  A
+// layer of up to 131072 scores is selected like a head, by one cluster (28
+// layers of 32736 scores: 15 us, against 40 us for the eight launches of the
+// layer select, whose digits each cross L2 between grids); longer ones by the
+// layer select.
+static cudaError_t layer_select(float* S, int n_layers, int T, int k, int32_t* chosen, void* scratch, cudaStream_t s) {
+  FinalArgs g{};
+  g.N = T;
+  g.Tv = T;
+  g.budget = k;
+  g.n_keep = k;
+  g.S = S;
+  g.idx = chosen;
+  g.h_kv = 1;
+  g.n_units = n_layers;
+  const cudaError_t e = launch_finalize_cluster(g, n_layers, true, s);
+  return e == cudaErrorNotSupported ? launch_layer_select(S, n_layers, T, k, chosen, scratch, s) : e;
+}
+
 }  // namespace ecokv
 
 using namespace ecokv;
@@ -544,8 +563,8 @@ ecokv_status ecokv_evict_adaptive(const ecokv_params* p, ecokv_dtype dtype, cons
   a.k_layer = keep_all ? 0 : p->h_kv * (p->budget - p->window);
   a.keep_all = keep_all ? 1 : 0;
   if (!keep_all && a.k_layer > 0 &&
-      launch_layer_select(f.S, p->n_layers, p->h_kv * L.Tv, a.k_layer, reinterpret_cast<int32_t*>(w + L.chosen),
-                          w + L.lsel, s) != cudaSuccess)
+      layer_select(f.S, p->n_layers, p->h_kv * L.Tv, a.k_layer, reinterpret_cast<int32_t*>(w + L.chosen), w + L.lsel,
+                   s) != cudaSuccess)
     return ECOKV_ERR_CUDA;
   // 3. per-head lists and offsets, then the gather over each layer's
   //    [h_kv * N] rows

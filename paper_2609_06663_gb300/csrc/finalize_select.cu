@@ -39,39 +39,42 @@ __global__ void __launch_bounds__(256) compact_kernel(CompactArgs a) {
   gather_rows<T>(a, blockIdx.y, r0, r0 + rows, threadIdx.x, blockDim.x);
 }
 
+// First index of the ascending list ch[0 .. n) with ch[i] >= key, by a warp: 32
+// probes a step (a binary search is one L2 round trip per halving: fifteen of
+// them, 10 us, for a layer of 26 000 chosen positions; three this way).
+__device__ __forceinline__ int lower_bound_warp(const int32_t* ch, int n, int key, int lane) {
+  int lo = 0, hi = n;  // the answer lies in [lo, hi]
+  while (lo < hi) {
+    const int step = (hi - lo + 31) / 32, at = lo + step * (lane + 1) - 1;  // the last element of this lane's part
+    const bool below = at < hi && __ldcg(ch + at) < key;
+    const int parts = __popc(__ballot_sync(0xffffffffu, below));  // ascending: the leading lanes
+    const int next = lo + step * parts;
+    hi = min(hi, next + step - 1);
+    lo = next;
+  }
+  return lo;
+}
+
 // One CTA per (head, layer): the head's share of the layer's chosen positions
-// (a contiguous run of the ascending list, found by binary search), written
-// as positions in the head, then its window; the head's list starts at the
+// (a contiguous run of the ascending list, found by search), written as
+// positions in the head, then its window; the head's list starts at the
 // number of chosen positions of lower heads plus their windows.
 __global__ void __launch_bounds__(256) adaptive_split_kernel(AdaptArgs a) {
-  const int h = blockIdx.x, l = blockIdx.y;
-  __shared__ int s_lo, s_hi;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int h = blockIdx.x, l = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ int s_at[2];
   const int32_t* ch = a.chosen + (size_t)l * a.k_layer;
-  if (threadIdx.x == 0) {
-    if (a.keep_all) {
-      s_lo = h * a.Tv;
-      s_hi = (h + 1) * a.Tv;
-    } else {
-      // first index with ch[i] >= key, for key = h Tv and (h + 1) Tv
-      int lo = 0, hi = a.k_layer;
-      while (lo < hi) {
-        const int m = (lo + hi) >> 1;
-        if (ch[m] < h * a.Tv) lo = m + 1; else hi = m;
-      }
-      s_lo = lo;
-      hi = a.k_layer;
-      while (lo < hi) {
-        const int m = (lo + hi) >> 1;
-        if (ch[m] < (h + 1) * a.Tv) lo = m + 1; else hi = m;
-      }
-      s_hi = lo;
-    }
+  if (warp < 2) {  // the head's first and last + 1
+    const int key = (h + warp) * a.Tv;
+    const int at = a.keep_all ? key : lower_bound_warp(ch, a.k_layer, key, lane);
+    if (lane == 0) s_at[warp] = at;
   }
   __syncthreads();
-  const int lo = s_lo, cnt = s_hi - s_lo, off = lo + h * a.W;
+  const int lo = s_at[0], cnt = s_at[1] - lo, off = lo + h * a.W;
   const size_t base = (size_t)l * a.h_kv * a.n_keep + off;
   for (int r = threadIdx.x; r < cnt + a.W; r += blockDim.x) {
-    const int pos = r < cnt ? (a.keep_all ? r : ch[lo + r] - h * a.Tv) : a.Tv + (r - cnt);
+    const int pos = r < cnt ? (a.keep_all ? r : __ldcg(ch + lo + r) - h * a.Tv) : a.Tv + (r - cnt);
     a.idx[base + r] = pos;
     a.src[base + r] = h * a.N + pos;
   }
@@ -137,8 +140,16 @@ cudaError_t launch_value_norms(const void* V, ecokv_dtype dt, int U, int N, int 
 }
 
 cudaError_t launch_adaptive_split(const AdaptArgs& a, int n_layers, cudaStream_t s) {
-  adaptive_split_kernel<<<dim3(a.h_kv, n_layers), 256, 0, s>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(a.h_kv, n_layers);
+  cfg.blockDim = dim3(256, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, adaptive_split_kernel, a);
 }
 
 // Scores of every unit and, with do_select, their top-k.
