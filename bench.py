@@ -94,8 +94,9 @@ def tensor_path(w) -> bool:
 
 def row_groups(w) -> int:
     """Launches of the tensor-core kernel per call: one per group of at most
-    120 window rows (g * W rows per head)."""
-    return (w.group * w.window + 119) // 120
+    120 window rows (g * W rows per head), or 128 past 64 MB of keys."""
+    most = 128 if w.units * w.n * w.d * 2 > 64 << 20 else 120
+    return (w.group * w.window + most - 1) // most
 
 
 SMS = 152  # of a GB300

@@ -42,8 +42,8 @@
  *  - Inputs must be finite; scores of non-finite inputs are unspecified.
  *  - Paths: bf16 inputs with n >= 128 stream K through a persistent
  *    tensor-core kernel, one launch for both of its passes over K, or one
- *    launch per group of at most 120 window rows when (h_q / h_kv) * window
- *    exceeds 120 (each group reads K twice); a few short heads (up to 64
+ *    launch per group of at most 120 window rows (128 past 64 MB of keys) when
+ *    (h_q / h_kv) * window exceeds that (each group reads K twice); a few short heads (up to 64
  *    window rows, one cluster of CTAs per head holding all its keys, every
  *    head's on the device at once: up to 10240 keys for 7 heads, 5120 for 19,
  *    640 for 152; no variant flag but the centroid's and the MixKV sign, the default

@@ -6,7 +6,7 @@
 // scores and the selection together (tc_short.cu, one launch); other bf16
 // inputs with n >= 128 stream K through the persistent tensor-core kernel
 // (tc_pass.cu, one launch for both passes, or one launch per group of at most
-// 120 window rows when (h_q/h_kv)*W exceeds 120);
+// 120 window rows, 128 past 64 MB of keys, when (h_q/h_kv)*W exceeds that);
 // fp32 inputs, other shapes and calls with ECOKV_FLAG_FORCE_SIMT use the
 // CUDA-core passes (score_simt.cu, two launches).  Either way one more launch
 // (finalize_select.cu) turns the pass-2 outputs into scores, selects and
@@ -72,16 +72,24 @@ static ecokv_status check_ws(const ecokv_params* p, void* ws, size_t ws_bytes) {
   return ECOKV_OK;
 }
 
-// Window rows per launch of the tensor-core kernel: all R of a unit when
-// R <= 120 (the MMA's N holds the rows padded to four plus eight statistics
-// columns, at most 128), else R split into ceil(R / 120) near-equal groups.
-static int tc_groups(int R) { return (R + 119) / 120; }
-static int tc_group_rows(int R) { return (R + tc_groups(R) - 1) / tc_groups(R); }
+// Window rows per launch of the tensor-core kernel: all R of a unit up to 120,
+// past that near-equal groups, each of which reads K twice.  Keys past about
+// half of L2 come from DRAM every time, so there a launch takes up to 128 rows
+// (8 heads x 131072 keys, R = 128: 135 us in one launch, 196 in two of 64 rows).
+static int tc_groups(const ecokv_params& p, int R) {
+  const long long key_bytes = (long long)p.n_layers * p.h_kv * p.n * kD * 2;
+  const int most = key_bytes > (64LL << 20) ? 128 : 120;
+  return (R + most - 1) / most;
+}
+static int tc_group_rows(const ecokv_params& p, int R) {
+  const int g = tc_groups(p, R);
+  return (R + g - 1) / g;
+}
 
 static bool use_tensor_path(const ecokv_params& p, ecokv_dtype dt) {
   if (dt != ECOKV_BF16 || (p.flags & ECOKV_FLAG_FORCE_SIMT)) return false;
   if (p.n < 128) return false;
-  return tc_rows(tc_group_rows((p.h_q / p.h_kv) * p.window)) > 0;
+  return tc_rows(tc_group_rows(p, (p.h_q / p.h_kv) * p.window)) > 0;
 }
 
 // Stage events of this host thread (ecokv_set_stage_events), recorded on the
@@ -215,7 +223,7 @@ static ecokv_status run_tc_group(const ecokv_params& p, const Layout& L, const v
 
 static ecokv_status run_tc_passes(const ecokv_params& p, const void* K, const void* Q, char* ws, cudaStream_t s) {
   const Layout L = make_layout(p, tc_records(p));
-  const int Rg = tc_group_rows(L.R);
+  const int Rg = tc_group_rows(p, L.R);
   for (int row0 = 0; row0 < L.R; row0 += Rg) {
     const int rows = L.R - row0 < Rg ? L.R - row0 : Rg;
     const ecokv_status st = run_tc_group(p, L, K, Q, ws, row0, rows, Rg, s);

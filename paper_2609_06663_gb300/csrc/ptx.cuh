@@ -165,6 +165,11 @@ __device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
+__device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 __device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
   return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);
 }
@@ -254,6 +259,14 @@ __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[N]) {
   if constexpr (n16 > n32) tmem_ld_x16(taddr + n32, r + n32);
   if constexpr (n8 > n16) tmem_ld_x8(taddr + n16, r + n16);
   if constexpr (N > n8) tmem_ld_x4(taddr + n8, r + n8);
+}
+
+// After tmem_wait_ld: values loaded before it are not used before it (the
+// compiler sees the loads' results as ready at once).
+template <int N>
+__device__ __forceinline__ void tmem_landed(uint32_t (&r)[N]) {
+#pragma unroll
+  for (int c = 0; c < N; ++c) asm volatile("" : "+r"(r[c]));
 }
 
 // Shared-memory matrix descriptor (tcgen05 format): start address, leading

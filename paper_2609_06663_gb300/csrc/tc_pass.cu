@@ -91,6 +91,9 @@ struct Cfg {
   static constexpr int kGroups = RP > 64 ? 2 : 3;              // tile groups of four warps
   static constexpr int kTileThreads = 128 * kGroups, kTileWarps = 4 * kGroups;
   static constexpr int kThreads = kCtl + kTileThreads;
+  // past 64 rows the stats warps, idle in pass 1, compute its key norms and sum
+  // weights; below, the rows leave the tile groups the time
+  static constexpr bool kStatNorms = RP > 64;
   // registers a thread: at launch, and after the split between the
   // warpgroups (tile groups hold a pass-1 sum per row and the columns in work)
   static constexpr uint32_t kRegsLaunch = RP > 64 ? 128 : 96;
@@ -100,7 +103,7 @@ struct Cfg {
                 "register split exceeds the launch's");
   static constexpr int kNP = (RP + kStatRows + 15) / 16 * 16;  // MMA N: window rows, then the statistics rows
   static constexpr int kCW = RP <= 32 ? RP : (RP == 56 ? 28 : (RP == 112 ? 56 : 32));  // columns read at once in pass 1
-  static constexpr int kS = RP > 56 ? (RP > 112 ? 3 : 4) : 5;  // key-tile stages
+  static constexpr int kS = RP > 56 ? 4 : 5;                    // key-tile stages
   static constexpr int kIQ = RP <= 16 ? 4 : (RP <= 32 ? 3 : 2);  // items in flight
   static constexpr int kNB = kNP <= 112 ? 4 : 3;               // TMEM accumulators
   static constexpr int kRed = RP > 64 ? 1 : 2;                 // pass-1 items whose row sums are held
@@ -325,6 +328,22 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = s.tmem_base;
   bool ok = true;
+  // a pass-1 tile's key kk (position i), the tile landed: its norm and sum
+  // weights, then this warp's share of the stage's release
+  auto key_work = [&](uint32_t stage, int kk, int i) {
+    if (sums) {
+      const float n2 = key_norm2(s.ktile[stage], kk);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&s.empty[stage]);  // done with the key tile
+      put_weights(s.wbuf[stage][0], kk, n2, i < a.N, a.kbar_n < a.N, i < a.kbar_n);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&s.wready[stage]);
+    } else {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&s.empty[stage]);
+    }
+  };
 
   if (warp >= kCtl / 32) {
     // ------------------------------------------------ tile groups (warps 8..)
@@ -362,17 +381,9 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
           const uint32_t stage = tc % kS, sph = (tc / kS) & 1u, b = tc % kNB, tph = (tc / kNB) & 1u;
           const int it0 = i0 + (int)t * kTile, i = it0 + kk;
           const bool valid = i < a.N;
-          if (!(ok = wait_warp(&s.full[stage], sph, a, 22u))) break;
-          if (sums) {
-            const float n2 = key_norm2(s.ktile[stage], kk);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&s.empty[stage]);  // done with the key tile
-            put_weights(s.wbuf[stage][0], kk, n2, valid, a.kbar_n < a.N, i < a.kbar_n);
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&s.wready[stage]);
-          } else if (lane == 0) {
-            mbar_arrive(&s.empty[stage]);
+          if (!C::kStatNorms) {
+            if (!(ok = wait_warp(&s.full[stage], sph, a, 22u))) break;
+            key_work(stage, kk, i);
           }
           if (!(ok = wait_warp(&s.tmem_full[b], tph, a, 12u))) break;
           tc_fence_after();
@@ -434,20 +445,15 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
           // columns after them: k . kbar in three terms, k . mu in two
           const uint32_t tb = tl + b * (uint32_t)kNP;
           float vp[4] = {0.f, 0.f, 0.f, 0.f};
+          const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
           constexpr int kCW = RP % 32 == 0 ? 32 : (RP % 28 == 0 ? 56 : RP);
 #pragma unroll
           for (int c0 = 0; c0 < RP; c0 += kCW) {
             uint32_t rc[kCW];
             tmem_ld<kCW>(tb + (uint32_t)c0, rc);
             tmem_wait_ld();
-#pragma unroll
-            for (int c = 0; c < kCW; c += 4) {
-              const float4 nl = *reinterpret_cast<const float4*>(nlse + c0 + c);
-              vp[0] += ex2(fmaf(__uint_as_float(rc[c]), a.scale_log2, nl.x));
-              vp[1] += ex2(fmaf(__uint_as_float(rc[c + 1]), a.scale_log2, nl.y));
-              vp[2] += ex2(fmaf(__uint_as_float(rc[c + 2]), a.scale_log2, nl.z));
-              vp[3] += ex2(fmaf(__uint_as_float(rc[c + 3]), a.scale_log2, nl.w));
-            }
+            tmem_landed(rc);
+            vote_rows<kCW>(rc, nlse + c0, scale2, vp);
           }
           uint32_t st[8];
           tmem_ld<8>(tb + (uint32_t)RP, st);
@@ -523,6 +529,8 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
     reg_dealloc<C::kRegsStats>();
     const int t = threadIdx.x - 128;
     uint32_t qpar = 0u;    // per slot: parity of the next qfull phase (completed by P1 and P2 items)
+    uint32_t tcnt = 0;     // tiles of the items so far
+    bool after_p2 = false;
     uint32_t sphase = 0u;  // of statbar, the bounded barrier among the four warps
     auto stat_sync = [&]() -> bool {
       __syncwarp();
@@ -537,6 +545,23 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
       ItemDesc<RP>& d = s.desc[slot];
       const int type = d.type, u = d.u;
       if (type == kExit) break;
+      const uint32_t ntiles = (uint32_t)d.ntiles;
+      if (C::kStatNorms && type == kP1) {
+        // (a stage's phase may only be waited for once the one before it is
+        // complete: after pass-2 tiles, which these warps do not wait for,
+        // the ring's last tiles first; they are all issued by now)
+        if (after_p2)
+          for (uint32_t q = tcnt > (uint32_t)kS ? tcnt - kS : 0u; q < tcnt && ok; ++q)
+            ok = wait_warp(&s.full[q % kS], (q / kS) & 1u, a, 24u);
+        after_p2 = false;
+        for (uint32_t q = tcnt; q < tcnt + ntiles && ok; ++q)
+          if ((ok = wait_warp(&s.full[q % kS], (q / kS) & 1u, a, 25u)))
+            key_work(q % kS, t, d.i0 + (int)(q - tcnt) * kTile + t);
+        if (!ok) break;
+      } else if (type == kP2) {
+        after_p2 = true;
+      }
+      tcnt += ntiles;
       if (type == kP2) {
         int c0, nrec;
         unit_slices(a, u, c0, nrec);

@@ -326,19 +326,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int t = grp + kGroups * j;
       if (t >= nt) break;
       float vp[4] = {0.f, 0.f, 0.f, 0.f};
+      const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
 #pragma unroll
       for (int c0 = 0; c0 < RP; c0 += SC::kCW) {
         uint32_t rc[SC::kCW];
         tmem_ld<SC::kCW>(tl + (uint32_t)(t * SC::kNQ + c0), rc);
         tmem_wait_ld();
-#pragma unroll
-        for (int c = 0; c < SC::kCW; c += 4) {
-          const float4 nl = *reinterpret_cast<const float4*>(nlse + c0 + c);
-          vp[0] += ex2(fmaf(__uint_as_float(rc[c]), a.scale_log2, nl.x));
-          vp[1] += ex2(fmaf(__uint_as_float(rc[c + 1]), a.scale_log2, nl.y));
-          vp[2] += ex2(fmaf(__uint_as_float(rc[c + 2]), a.scale_log2, nl.z));
-          vp[3] += ex2(fmaf(__uint_as_float(rc[c + 3]), a.scale_log2, nl.w));
-        }
+        tmem_landed(rc);
+        vote_rows<SC::kCW>(rc, nlse + c0, scale2, vp);
       }
       const float v = (vp[0] + vp[1]) + (vp[2] + vp[3]);
       wait(&s.stat, 45u);

@@ -111,6 +111,33 @@ __device__ __forceinline__ void combine_maxsum(float& m, float& z, float m2, flo
   m = M;
 }
 
+// (x, y) <- (x, y) * s + (a, b) as one packed operation, x and y as float bits
+__device__ __forceinline__ void fma_pair(uint32_t& x, uint32_t& y, uint64_t s, float a, float b) {
+  const uint64_t r = ffma2((uint64_t)x | (uint64_t)y << 32, s, pack_f32x2(a, b));
+  x = (uint32_t)r;
+  y = (uint32_t)(r >> 32);
+}
+// (x, y) <- (x, y) + (a, b) as one packed operation
+__device__ __forceinline__ void add_pair(float& x, float& y, float a, float b) {
+  const uint64_t r = fadd2(pack_f32x2(x, y), pack_f32x2(a, b));
+  x = f32x2_lo(r);
+  y = f32x2_hi(r);
+}
+
+// The vote of a key: the sum over kN rows of 2^(x scale - lse), x the logits and
+// nlse the negated log2-sum-exp (16-byte aligned).
+template <int kN>
+__device__ __forceinline__ void vote_rows(uint32_t (&rc)[kN], const float* nlse, uint64_t scale2, float (&vp)[4]) {
+#pragma unroll
+  for (int c = 0; c < kN; c += 4) {
+    const float4 nl = *reinterpret_cast<const float4*>(nlse + c);
+    fma_pair(rc[c], rc[c + 1], scale2, nl.x, nl.y);
+    fma_pair(rc[c + 2], rc[c + 3], scale2, nl.z, nl.w);
+    add_pair(vp[0], vp[1], ex2(__uint_as_float(rc[c])), ex2(__uint_as_float(rc[c + 1])));
+    add_pair(vp[2], vp[3], ex2(__uint_as_float(rc[c + 2])), ex2(__uint_as_float(rc[c + 3])));
+  }
+}
+
 // Sum of v[j] over the lanes of a warp for every j < N, scattered: five
 // halving steps leave lane l with the rows base .. base + kOut - 1 below lim.
 template <int N>
@@ -150,16 +177,19 @@ struct ScatterSum {
 // kept.  vis_from: a row with window position j sees the lane's key iff j >=
 // vis_from (INT_MAX for a key past N); j0: the first row's window position.
 // The columns are read kCW at a time: a read costs about 0.25 us whatever its
-// width (in eights, 56 rows took 2.3 us a tile).
+// width (in eights, 56 rows took 2.3 us a tile; 128 rows in sixteens, each read
+// issued while the columns before it were worked on, 18 % longer than in 32s).
 template <int RP, int kCW>
 __device__ __forceinline__ void pass1_rows(uint32_t taddr, float (&z)[RP], float* ref, float scale, bool first,
                                            bool all_vis, int vis_from, int j0, int W, int lane, uint64_t* bar_empty) {
   int jw = j0;
+  const uint64_t scale2 = pack_f32x2(scale, scale);
 #pragma unroll
   for (int c0 = 0; c0 < RP; c0 += kCW) {
     uint32_t rc[kCW];
     tmem_ld<kCW>(taddr + (uint32_t)c0, rc);
     tmem_wait_ld();
+    tmem_landed(rc);
     if (c0 + kCW == RP) {
       tc_fence_before();
       __syncwarp();
@@ -182,10 +212,8 @@ __device__ __forceinline__ void pass1_rows(uint32_t taddr, float (&z)[RP], float
 #pragma unroll
       for (int c = 0; c < kCW; c += 4) {
         const float4 nr = *reinterpret_cast<const float4*>(ref + c0 + c);
-        rc[c] = __float_as_uint(fmaf(__uint_as_float(rc[c]), scale, nr.x));
-        rc[c + 1] = __float_as_uint(fmaf(__uint_as_float(rc[c + 1]), scale, nr.y));
-        rc[c + 2] = __float_as_uint(fmaf(__uint_as_float(rc[c + 2]), scale, nr.z));
-        rc[c + 3] = __float_as_uint(fmaf(__uint_as_float(rc[c + 3]), scale, nr.w));
+        fma_pair(rc[c], rc[c + 1], scale2, nr.x, nr.y);
+        fma_pair(rc[c + 2], rc[c + 3], scale2, nr.z, nr.w);
       }
       if (!all_vis) {
 #pragma unroll
@@ -209,7 +237,8 @@ __device__ __forceinline__ void pass1_rows(uint32_t taddr, float (&z)[RP], float
         }
       }
 #pragma unroll
-      for (int c = 0; c < kCW; ++c) z[c0 + c] += ex2(__uint_as_float(rc[c]));
+      for (int c = 0; c < kCW; c += 2)
+        add_pair(z[c0 + c], z[c0 + c + 1], ex2(__uint_as_float(rc[c])), ex2(__uint_as_float(rc[c + 1])));
     }
   }
   __syncwarp();

@@ -41,3 +41,11 @@ def test_logits_that_outgrow_their_reference(group, window):
     check_scores(S[0, 0].cpu().double().numpy(), r, TOL["bf16"], "growing keys")
     check_selection(idx[0, 0].cpu().numpy(), r, op, TOL["bf16"], "growing keys")
     assert abs(float(lam[0, 0]) - r["lam"]) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("group,window", [(4, 32), (8, 16), (8, 32)], ids=lambda v: str(v))
+def test_128_rows_in_one_launch(group, window):
+    # more than 64 MB of keys: up to 128 window rows a launch (256 rows: two),
+    # the odd last tile with keys that not every row sees
+    run_and_compare(small_workload(33001, h_kv=8, group=group, window=window, budget=3300, dtype="bf16", seed=6),
+                    units=[(0, 0), (0, 7)])
