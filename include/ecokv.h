@@ -272,8 +272,9 @@ ecokv_status ecokv_evict_noalloc(const ecokv_params* p, ecokv_dtype dtype, const
  *                    K and Qwin and the indices.
  * Data movement, in stream order: K and Qwin are copied to the workspace once
  * (both streaming passes read them there); the gather reads the kept V rows
- * and writes K_out / V_out directly in host memory, so V crosses the host
- * link only for the kept rows; idx is copied back at the end.  Per call the
+ * and writes K_out, V_out and idx directly in host memory (idx by a copy at
+ * the end where its address is not a multiple of 4), so V crosses the host
+ * link only for the kept rows.  Per call the
  * host link carries |K| + |Qwin| + B/n of |V| inbound and |K_out| + |V_out| +
  * |idx| outbound, against |K| + |V| + |Qwin| inbound for ecokv_evict on
  * copied inputs.  Exception: with ECOKV_FLAG_VNORM_IMP the value norms are

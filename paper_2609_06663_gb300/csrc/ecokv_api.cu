@@ -590,7 +590,8 @@ ecokv_status ecokv_evict_adaptive(const ecokv_params* p, ecokv_dtype dtype, cons
 
 static ecokv_status evict_impl(const ecokv_params* p, ecokv_dtype dtype, const void* K, const void* V,
                                const void* Qwin, int32_t* idx, void* K_out, void* V_out, float* S, float* lambda,
-                               void* ws, size_t ws_bytes, void* stream, const int32_t* layer_budget) {
+                               void* ws, size_t ws_bytes, void* stream, const int32_t* layer_budget, bool host = false,
+                               int32_t* idx_out = nullptr) {
   ecokv_status st = ecokv_check_params(p);
   if (st != ECOKV_OK) return st;
   if (dtype != ECOKV_F32 && dtype != ECOKV_BF16) return ECOKV_ERR_INVALID_ARG;
@@ -610,6 +611,8 @@ static ecokv_status evict_impl(const ecokv_params* p, ecokv_dtype dtype, const v
   f.lambda = lambda;
   f.idx = idx;
   CompactArgs c = compact_args(*p, K, V, idx, K_out, V_out, reinterpret_cast<unsigned*>(w + L.status));
+  c.host = host ? 1 : 0;
+  c.idx_out = idx_out;
   if (layer_budget != nullptr) {
     f.n_lb = c.n_lb = p->n_layers;
     for (int l = 0; l < p->n_layers; ++l) {
@@ -711,3 +714,10 @@ const char* ecokv_status_string(ecokv_status s) {
 }
 
 }  // extern "C"
+
+ecokv_status ecokv::evict_host_rows(const ecokv_params* p, ecokv_dtype dtype, const void* K, const void* V,
+                                    const void* Qwin, int32_t* idx, int32_t* idx_out, void* K_out, void* V_out,
+                                    float* lambda, void* ws, size_t ws_bytes, void* stream) {
+  return evict_impl(p, dtype, K, V, Qwin, idx, K_out, V_out, nullptr, lambda, ws, ws_bytes, stream, nullptr, true,
+                    idx_out);
+}

@@ -126,6 +126,8 @@ struct CompactArgs {
   void* V_out;
   int N, n_keep;
   unsigned* status;  // may be null
+  int host;          // V and the outputs lie in host memory
+  int32_t* idx_out;  // host: a second copy of the indices, or null
   // per-layer budgets: unit u copies keep[u / h_kv] rows (of stride n_keep)
   int h_kv, n_lb;
   int keep[kMaxLayerBudgets];
@@ -169,5 +171,11 @@ cudaError_t launch_layer_select(const float* S, int n_layers, int T, int k, int3
 // (select_only: the top-k of the given scores f.S); cudaErrorNotSupported
 // when the unit is too long for one cluster.
 cudaError_t launch_finalize_cluster(const FinalArgs& f, int U, bool select_only, cudaStream_t s);
+
+// ecokv_evict for V, K_out, V_out and lambda in host memory; idx_out: a second,
+// host copy of the indices (4-byte aligned), or null.
+ecokv_status evict_host_rows(const ecokv_params* p, ecokv_dtype dtype, const void* K, const void* V, const void* Qwin,
+                             int32_t* idx, int32_t* idx_out, void* K_out, void* V_out, float* lambda, void* ws,
+                             size_t ws_bytes, void* stream);
 
 }  // namespace ecokv

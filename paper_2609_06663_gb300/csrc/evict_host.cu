@@ -1,12 +1,12 @@
 // ecokv_evict_host: the eviction pass for a KV cache resident in host memory
 // that the device addresses directly (pinned and mapped, unified addressing).
 //
-// Built on the public entry point: K and Qwin are copied once into the
-// workspace (both streaming passes read K, so one copy beats two trips over
-// the host link); ecokv_evict then runs on those copies with V, K_out, V_out
-// and lambda left in host memory, so that the gather reads only the kept V
-// rows over the link and writes the outputs there directly; the indices,
-// made in the workspace, are copied back last.  With value-norm importance
+// K and Qwin are copied once into the workspace (both streaming passes read K,
+// so one copy beats two trips over the host link); the pass then runs on those
+// copies with V, K_out, V_out and lambda left in host memory, so that the
+// gather reads only the kept V rows over the link and writes the outputs, and
+// the indices made in the workspace, there directly (the indices by a copy of
+// their own: 9 us).  With value-norm importance
 // (ECOKV_FLAG_VNORM_IMP) the norm kernel reads every row of V where it lies,
 // so then all of V crosses the link as well.
 //
@@ -78,8 +78,11 @@ extern "C" ecokv_status ecokv_evict_host(const ecokv_params* p, ecokv_dtype dtyp
   int32_t* idx_dev = reinterpret_cast<int32_t*>(w + h.idx_off);
   if (cudaMemcpyAsync(K_dev, K, h.k_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return ECOKV_ERR_CUDA;
   if (cudaMemcpyAsync(Q_dev, Qwin, h.q_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return ECOKV_ERR_CUDA;
-  st = ecokv_evict(p, dtype, K_dev, V, Q_dev, idx_dev, K_out, V_out, nullptr, lambda, ws, h.base, stream);
-  if (st != ECOKV_OK) return st;
+  // the gather writes the host's copy of the indices too (an odd address: a copy does)
+  const bool direct = ((uintptr_t)idx & 3u) == 0;
+  st = ecokv::evict_host_rows(p, dtype, K_dev, V, Q_dev, idx_dev, direct ? idx : nullptr, K_out, V_out, lambda, ws,
+                              h.base, stream);
+  if (st != ECOKV_OK || direct) return st;
   if (cudaMemcpyAsync(idx, idx_dev, h.idx_bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess) return ECOKV_ERR_CUDA;
   return ECOKV_OK;
 }

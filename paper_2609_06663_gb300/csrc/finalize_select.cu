@@ -39,6 +39,31 @@ __global__ void __launch_bounds__(256) compact_kernel(CompactArgs a) {
   gather_rows<T>(a, blockIdx.y, r0, r0 + rows, threadIdx.x, blockDim.x);
 }
 
+// The gather of a cache in host memory.  Bound by the host link: V's rows are
+// read over it, both tensors' rows and the indices are written over it.  One
+// block copies one tensor's rows, those of K (a device copy) before those of
+// V, so that K's rows cross the link while V's are still arriving; a block
+// that copies both keeps its writes until its reads have landed, and the two
+// directions follow each other (4 x 4 heads, 1024 kept rows: 65.5 -> 55.5 us;
+// 32 rows a block 1.5 us slower than 64).  In device memory the split is the
+// slower one (28 x 4 heads, 3277 rows: 63.5 against 69.6 us): a block there
+// copies both.
+constexpr int kHostRows = 64;
+
+template <typename T>
+__global__ void __launch_bounds__(256) compact_host_kernel(CompactArgs a) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int u = blockIdx.y, r0 = blockIdx.x * kHostRows, r1 = r0 + kHostRows;
+  if (blockIdx.z == 0) {
+    gather_rows_of<T>(a, a.K, a.K_out, u, r0, r1, threadIdx.x, blockDim.x);
+    if (a.idx_out != nullptr)
+      for (int r = r0 + threadIdx.x; r < min(r1, a.n_keep); r += blockDim.x)
+        a.idx_out[(size_t)u * a.n_keep + r] = __ldcg(a.idx + (size_t)u * a.n_keep + r);
+  } else {
+    gather_rows_of<T>(a, a.V, a.V_out, u, r0, r1, threadIdx.x, blockDim.x);
+  }
+}
+
 // First index of the ascending list ch[0 .. n) with ch[i] >= key, by a warp: 32
 // probes a step (a binary search is one L2 round trip per halving: fifteen of
 // them, 10 us, for a layer of 26 000 chosen positions; three this way).
@@ -178,7 +203,7 @@ cudaError_t launch_select(const FinalArgs& f, int U, cudaStream_t s) {
 cudaError_t launch_compact(const CompactArgs& a, ecokv_dtype dt, int U, cudaStream_t s) {
   if (a.n_keep == 0 || U == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((a.n_keep + 31) / 32, U);
+  cfg.gridDim = a.host ? dim3((a.n_keep + kHostRows - 1) / kHostRows, U, 2) : dim3((a.n_keep + 31) / 32, U);
   cfg.blockDim = dim3(256, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -186,6 +211,9 @@ cudaError_t launch_compact(const CompactArgs& a, ecokv_dtype dt, int U, cudaStre
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (a.host)
+    return dt == ECOKV_F32 ? cudaLaunchKernelEx(&cfg, compact_host_kernel<float>, a)
+                           : cudaLaunchKernelEx(&cfg, compact_host_kernel<__nv_bfloat16>, a);
   if (dt == ECOKV_F32) return cudaLaunchKernelEx(&cfg, compact_kernel<float>, a);
   return cudaLaunchKernelEx(&cfg, compact_kernel<__nv_bfloat16>, a);
 }

@@ -19,7 +19,8 @@
 //   ascending) (Sec. 3), by an MSB-first radix select on the order-preserving
 //   32-bit image of S, emitted in ascending position (warp ballots over
 //   contiguous ranges) and followed by the window.
-// gather_rows: K_out[r] = K[idx[r]], V_out[r] = V[idx[r]], 16-byte copies.
+// gather_rows: K_out[r] = K[idx[r]], V_out[r] = V[idx[r]], 16-byte copies;
+//   gather_rows_of: one of the two.
 #pragma once
 
 #include <math.h>
@@ -370,6 +371,38 @@ __device__ void gather_rows(const CompactArgs& a, int u, int r0, int r1, int tid
         __stcs(Ko + dst[j], kv[j]);
         __stcs(Vo + dst[j], vv[j]);
       }
+  }
+}
+
+// Copy rows [r0, r1) of unit u of one tensor: out[r] = in[idx[r]], four 16-byte
+// vectors in flight per thread.
+template <typename T>
+__device__ void gather_rows_of(const CompactArgs& a, const void* in, void* out, int u, int r0, int r1, int tid,
+                               int nt) {
+  constexpr int vpr = kD * sizeof(T) / 16;  // 16-byte vectors per row
+  const uint4* src = reinterpret_cast<const uint4*>(in) + (size_t)u * a.N * vpr;
+  uint4* dst = reinterpret_cast<uint4*>(out) + ((size_t)u * a.n_keep + r0) * vpr;
+  const int32_t* idx = a.idx + (size_t)u * a.n_keep + r0;
+  const int total = (min(r1, a.n_lb ? a.keep[u / a.h_kv] : a.n_keep) - r0) * vpr;
+  for (int e0 = tid; e0 < total; e0 += 4 * nt) {
+    uint4 x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int e = e0 + j * nt;
+      x[j] = make_uint4(0u, 0u, 0u, 0u);
+      if (e < total) {
+        const int i = __ldcg(idx + e / vpr);
+        if (i >= 0 && i < a.N) {
+          x[j] = __ldcs(src + (size_t)i * vpr + e % vpr);  // each row is read once
+        } else if (a.status != nullptr) {
+          atomicCAS(a.status, 0u, (unsigned)ECOKV_ERR_DEVICE_INDEX);
+          a.status[1] = (unsigned)u;
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (e0 + j * nt < total) __stcs(dst + e0 + j * nt, x[j]);
   }
 }
 
