@@ -158,7 +158,7 @@ def measured_peaks() -> tuple[float, str]:
 # The sources that define the streaming kernel and the parameters it is
 # launched with (item size, schedule lag, tail split): a recorded DRAM traffic
 # figure is valid while these are unchanged.
-STREAMING_SOURCES = ("tc_pass.cu", "tc_pass.cuh", "ptx.cuh", "finalize_select.cuh", "ecokv_internal.cuh",
+STREAMING_SOURCES = ("tc_pass.cu", "tc_pass.cuh", "tc_tile.cuh", "ptx.cuh", "finalize_select.cuh", "ecokv_internal.cuh",
                      "ecokv_api.cu")
 
 

@@ -286,8 +286,11 @@ static int short_ctas(const ecokv_params& p, ecokv_dtype dt) {
   if (!use_tensor_path(p, dt) || p.sched_wave != 0 || p.sched_lag != 0) return 0;
   if (p.flags & (ECOKV_FLAG_VNORM_IMP | ECOKV_FLAG_WINSOR_1 | ECOKV_FLAG_WINSOR_5 | ECOKV_FLAG_MAD | ECOKV_FLAG_TEST_STALL))
     return 0;
-  return short_cluster((p.h_q / p.h_kv) * p.window, (p.n + 127) / 128, (long long)p.n_layers * p.h_kv, num_sms());
+  const int C =
+      short_cluster((p.h_q / p.h_kv) * p.window, (p.n + 127) / 128, (long long)p.n_layers * p.h_kv, num_sms());
+  return C <= tc_records(p) ? C : 0;  // one pass-2 record per CTA of a unit
 }
+
 static ecokv_status run_short(const ecokv_params& p, const Layout& L, const void* K, const void* Q, char* ws,
                               const FinalArgs& f, int C, cudaStream_t s) {
   ShortArgs a{};

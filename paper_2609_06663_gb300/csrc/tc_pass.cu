@@ -22,9 +22,9 @@
 // waves of `uw` units in unit order; the tiles of a wave are cut into at most
 // P contiguous slices of near-equal length.  Wave w's slices are dealt to the
 // CTAs in a rotation that advances with w, so that the slices one tile longer
-// than others fall to different CTAs.  One item per unit a slice touches (pass 2 walks a slice backwards,
-// units and tiles, so that it starts with the keys pass 1 read last, the
-// likeliest still to be in L2).  Step s of a CTA holds the P1 items of its
+// than others fall to different CTAs.  One item per unit a slice touches
+// (pass 2 walks a slice backwards, units and tiles, so that it starts with the
+// keys pass 1 read last, the likeliest still to be in L2).  Step s of a CTA holds the P1 items of its
 // slice of wave s, then the P2 items of its slice of wave s - lag.  With one
 // wave (the default) all of pass 1 precedes pass 2.  Every CTA is resident,
 // so waits on other CTAs' items end.
@@ -49,8 +49,8 @@
 // P2 items.  The others are tile groups of four warps, one key per thread:
 // tile t goes to group t mod 3 (mod 2 past 64 window rows, whose pass-1 sums
 // take twice the registers), which computes the key norms and sum weights
-// from shared memory as the tile lands and then works through the tile's
-// logits in TMEM.  A tile costs a group about 1.5 us in pass 1 and 1 us in
+// from shared memory as the tile lands (past 64 rows the stats warps do so in
+// pass 1) and then works through the tile's logits in TMEM.  A tile costs a group about 1.5 us in pass 1 and 1 us in
 // pass 2, nearly all of it latency, so several tiles are in progress at once.
 // (With key norms and logits on separate sets of four and eight warps the
 // four key warps set pass 1's pace at 0.85 us per tile: 0.224 ms for 32 layers
