@@ -9,7 +9,7 @@ namespace ecokv {
 namespace {
 
 template <int kMode, int kSh, bool kVar>
-__global__ void __launch_bounds__(kCThreads, Shape<kSh>::kMinCtas) finalize_cluster_kernel(FinalArgs f) {
+__global__ void __launch_bounds__(Shape<kSh>::kThreads, Shape<kSh>::kMinCtas) finalize_cluster_kernel(FinalArgs f) {
   extern __shared__ __align__(16) uint8_t fc_smem[];
   ClusterSmem<kSh>& sm = *reinterpret_cast<ClusterSmem<kSh>*>(fc_smem);
   cg::cluster_group cl = cg::this_cluster();
@@ -45,7 +45,7 @@ template <int kSh>
 cudaError_t launch_shape(const FinalArgs& f, int U, int C, bool select_only, cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(U * C), 1, 1);
-  cfg.blockDim = dim3(kCThreads, 1, 1);
+  cfg.blockDim = dim3(Shape<kSh>::kThreads, 1, 1);
   cfg.dynamicSmemBytes = sizeof(ClusterSmem<kSh>);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
@@ -69,7 +69,40 @@ cudaError_t launch_shape(const FinalArgs& f, int U, int C, bool select_only, cud
 // Per device: the attributes set, and whether clusters of 16 CTAs of the
 // longest shape can be resident (cudaOccupancyMaxActiveClusters > 0).
 std::atomic<int> g_setup[64];  // 0 = not yet, 1 = set, clusters of 16 unavailable, 2 = set and available
-std::atomic<int> g_sms[64];    // SMs, set before g_setup
+// Clusters of C CTAs of shapes 0-3 resident at once plus one, at [shape][C - 1]; 0 = not asked yet.
+std::atomic<int> g_fit[64][4][16];
+
+// Clusters of C CTAs that the current device holds at once (the occupancy
+// query's answer, asked once; a racing thread asks again).
+template <int kSh>
+int clusters_fit(int dev, int C) {
+  int n = g_fit[dev][kSh][C - 1].load();
+  if (n > 0) return n - 1;
+  n = 0;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)C * 1024u, 1, 1);
+  cfg.blockDim = dim3(Shape<kSh>::kThreads, 1, 1);
+  cfg.dynamicSmemBytes = sizeof(ClusterSmem<kSh>);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&n, (const void*)finalize_cluster_kernel<1, kSh, false>, &cfg) != cudaSuccess) {
+    cudaGetLastError();  // an unavailable configuration leaves no error behind
+    n = 0;
+  }
+  g_fit[dev][kSh][C - 1].store(n + 1);
+  return n;
+}
+
+int clusters_fit(int dev, int sh, int C) {
+  return sh == 0 ? clusters_fit<0>(dev, C) : sh == 1 ? clusters_fit<1>(dev, C)
+                                         : sh == 2   ? clusters_fit<2>(dev, C)
+                                                     : clusters_fit<3>(dev, C);
+}
 
 int device_setup() {
   int dev = 0;
@@ -77,60 +110,52 @@ int device_setup() {
   int st = g_setup[dev].load();
   if (st != 0) return st;
   if (set_attrs<0>(false) != cudaSuccess || set_attrs<1>(false) != cudaSuccess || set_attrs<2>(false) != cudaSuccess ||
-      set_attrs<3>(false) != cudaSuccess)
+      set_attrs<3>(false) != cudaSuccess || set_attrs<5>(false) != cudaSuccess)
     return -1;
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return -1;
-  g_sms[dev].store(sms);
-  st = 1;
-  if (set_attrs<0>(true) == cudaSuccess && set_attrs<3>(true) == cudaSuccess) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(16u * 16u, 1, 1);
-    cfg.blockDim = dim3(kCThreads, 1, 1);
-    cfg.dynamicSmemBytes = sizeof(ClusterSmem<3>);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 16;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (const void*)finalize_cluster_kernel<1, 3, false>, &cfg) == cudaSuccess &&
-        n > 0)
-      st = 2;
-  }
+  const bool wide = set_attrs<0>(true) == cudaSuccess && set_attrs<3>(true) == cudaSuccess;
+  st = wide && clusters_fit<3>(dev, 16) > 0 ? 2 : 1;
   cudaGetLastError();  // an unavailable configuration leaves no error behind
   g_setup[dev].store(st);
   return st;
 }
 
 // Shape and cluster size for U units of Tv candidates; shape -1 when none takes
-// them.  The fewest candidates a thread whose CTAs are all resident at once;
-// failing that (many units) the fewest in clusters of at most four.  One layer
-// of 4 heads x 32768 keys: 16 CTAs of 8 a thread 15 us, 4 of 32 a thread 25 us;
-// 28 layers x 4 heads of that length: 3 waves of the former, one of the latter.
-void pick_shape(int Tv, long long U, int long_ok, int sms, int& sh, int& C) {
+// them.  The fewest candidates a thread whose clusters are all resident at once
+// (one layer of 4 heads x 32768 keys: 16 CTAs of 8 a thread 15 us, 4 of 32 a
+// thread 25 us; 28 layers x 4 heads of that length: 3 waves of the former, one
+// of the latter).  Failing that (many units) clusters of at most four: of
+// 128-thread CTAs up to 8192 candidates, seven to an SM (32 x 32 heads of 2048
+// keys: 21 us against 27 in CTAs of 256 threads, 608 at once; 20 x 32 of 6000
+// keys 42 against 53), else the fewest candidates a thread.  The 128-thread
+// CTAs in clusters of more than four, resident at once, lost to 32 candidates a
+// thread (28 x 4 heads of 16411 keys, nine CTAs each: 234 against 218 us a
+// call).  What is resident is the occupancy query's answer: by the SM count
+// alone, 112 clusters of four at three CTAs an SM would fit, but the SMs of a
+// GPC hold whole clusters only (28 x 4 heads of 14500 keys: 202 us a call in
+// two waves of those, 194 in one of 32 candidates a thread).
+void pick_shape(int Tv, long long U, int dev, bool long_ok, int& sh, int& C) {
   const int t = Tv > 0 ? Tv : 1;
   const int cap[4] = {Shape<0>::kCap, Shape<1>::kCap, Shape<2>::kCap, Shape<3>::kCap};
   const int most[4] = {long_ok ? Shape<0>::kMaxCluster : 8, Shape<1>::kMaxCluster, Shape<2>::kMaxCluster,
                        long_ok ? Shape<3>::kMaxCluster : 8};
-  const int resident[4] = {Shape<0>::kMinCtas, Shape<1>::kMinCtas, Shape<2>::kMinCtas, Shape<3>::kMinCtas};
   for (sh = 0; sh < 4; ++sh) {
     C = (t + cap[sh] - 1) / cap[sh];
-    if (C <= most[sh] && U * C <= (long long)resident[sh] * sms) return;
+    if (C <= most[sh] && U <= clusters_fit(dev, sh, C)) return;
   }
-  for (sh = 0; sh < 4; ++sh) {
+  sh = 5;
+  C = (t + Shape<5>::kCap - 1) / Shape<5>::kCap;
+  if (C <= Shape<5>::kMaxCluster) return;
+  for (sh = 1; sh < 4; ++sh) {
     C = (t + cap[sh] - 1) / cap[sh];
-    if (C <= (sh < 3 ? 4 : most[3])) return;
+    if (C <= most[sh]) return;
   }
   sh = -1;
   C = 0;
 }
 
-int current_sms() {
+int current_device() {
   int dev = 0;
-  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_sms[dev].load() : 0;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? dev : 0;
 }
 
 }  // namespace
@@ -139,7 +164,7 @@ bool cluster_finalize_fits(int Tv) {
   const int st = device_setup();
   if (st < 0) return false;
   int sh, C;
-  pick_shape(Tv, 1, st == 2, current_sms(), sh, C);
+  pick_shape(Tv, 1, current_device(), st == 2, sh, C);
   return sh >= 0;
 }
 
@@ -147,12 +172,13 @@ cudaError_t launch_finalize_cluster(const FinalArgs& f, int U, bool select_only,
   const int st = device_setup();
   if (st < 0) return cudaErrorUnknown;
   int sh, C;
-  pick_shape(f.Tv, U, st == 2, current_sms(), sh, C);
+  pick_shape(f.Tv, U, current_device(), st == 2, sh, C);
   switch (sh) {
     case 0: return launch_shape<0>(f, U, C, select_only, s);
     case 1: return launch_shape<1>(f, U, C, select_only, s);
     case 2: return launch_shape<2>(f, U, C, select_only, s);
     case 3: return launch_shape<3>(f, U, C, select_only, s);
+    case 5: return launch_shape<5>(f, U, C, select_only, s);
   }
   return cudaErrorNotSupported;
 }

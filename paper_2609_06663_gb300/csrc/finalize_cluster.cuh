@@ -4,14 +4,16 @@
 // with the cluster-wide reductions done through distributed shared memory.
 //
 // Shapes: 8, 16 or 32 candidates a thread and up to 16, 4 or 4 CTAs, or 32 a
-// thread and up to 16 CTAs (units of up to 131072 candidates).  The kernel is
-// all latency, and shorter the less a thread has to do, so a unit is spread as
-// widely as leaves every unit's CTAs resident at once (three or four per SM):
-// four heads of 32760 candidates on 16 CTAs each, the 112 units of a prefill
-// (28 layers x 4 KV heads) of that length on four each.
+// thread and up to 16 CTAs (units of up to 131072 candidates), of 256 threads;
+// and 16 a thread in up to 4 CTAs of 128 threads.  The kernel is all latency,
+// and shorter the less a thread has to do, so a unit is spread as widely as
+// leaves every unit's CTAs resident at once (three or four per SM): four heads
+// of 32760 candidates on 16 CTAs each, the 112 units of a prefill (28 layers x
+// 4 KV heads) of that length on four each.  Past that, for the many heads of a
+// prefill without grouped queries, the small CTAs run in the fewest waves.
 //
 // CTA rank r of the cluster owns candidates [r * cap, (r + 1) * cap) of the
-// unit (cap = 256 threads x kJ); thread t of it owns the kJ consecutive
+// unit (cap = the CTA's threads x kJ); thread t of it owns the kJ consecutive
 // candidates from r * cap + kJ * t and keeps their pooled importance, then
 // the keys of their scores, in registers.  The raw votes of the CTA (with the
 // pooling halo) are staged in shared memory with one pad word after every 32,
@@ -54,21 +56,23 @@ namespace cg = cooperative_groups;
 
 namespace ecokv {
 
-constexpr int kCThreads = 256;
-constexpr int kCWarps = kCThreads / 32;
+constexpr int kCThreads = 256;  // of a CTA, but for the small one's 128
 constexpr int kHalo = 16;  // pooling halo kept in shared memory (kernel <= 33)
 
 // Shapes (kSh), see above: candidates a thread, CTAs a unit, histogram ranges
 // (their 16-bit counts of every rank take the place of the staged scores).
-// Shape 4 is the short-unit kernel's: a CTA's keys are at most 640.
+// Shape 4 is the short-unit kernel's: a CTA's keys are at most 640.  Shape 5 is
+// the small CTA's.
 template <int kSh>
 struct Shape {
-  static constexpr int kJ = kSh == 4 ? 4 : (kSh == 0 ? 8 : (kSh == 1 ? 16 : 32));  // candidates a thread owns
-  static constexpr int kCap = kCThreads * kJ;                     // candidates a CTA owns
-  static constexpr int kMaxCluster = kSh == 1 || kSh == 2 ? 4 : 16;              // CTAs a unit may take
+  static constexpr int kThreads = kSh == 5 ? 128 : kCThreads, kWarps = kThreads / 32;
+  // candidates a thread owns
+  static constexpr int kJ = kSh == 4 ? 4 : (kSh == 0 ? 8 : (kSh == 1 || kSh == 5 ? 16 : 32));
+  static constexpr int kCap = kThreads * kJ;                      // candidates a CTA owns
+  static constexpr int kMaxCluster = kSh == 1 || kSh == 2 || kSh == 5 ? 4 : 16;  // CTAs a unit may take
   static constexpr int kQ = kCap + 2 * kHalo;                     // staged raw votes
   static constexpr int kBins = kSh == 1 || kSh == 2 ? 2048 : 1024;
-  static constexpr int kMinCtas = kSh == 1 ? 3 : 4;               // resident CTAs per SM asked of the compiler
+  static constexpr int kMinCtas = kSh == 5 ? 7 : (kSh == 1 ? 3 : 4);  // resident CTAs per SM asked of the compiler
   static constexpr bool kAlias = kSh != 4;                        // histograms in the place of the staged scores
 };
 constexpr int kList = 512;  // keys ranked directly
@@ -98,15 +102,16 @@ struct ClusterSmem {
   float4 ext_all[Sh::kMaxCluster];
   double simp_all[Sh::kMaxCluster];  // value-norm importance: every rank's sum of S_imp
   double wsum_all[Sh::kMaxCluster];  // winsorised min-max / MAD scaling: every rank's sum of s_E terms
-  float red[kCWarps][8];  // per-warp partials
-  alignas(16) float4 red4[kCWarps];   // per-warp extrema
+  float red[Shape<kSh>::kWarps][8];  // per-warp partials
+  alignas(16) float4 red4[Shape<kSh>::kWarps];   // per-warp extrema
   float edge[32];         // pooling edge values
   float sc[8];            // broadcast scalars
   double dsc[2];          // sums behind the means of S_imp and of S_div
-  double dred[kCWarps];   // per-warp sums of S_imp (value-norm importance)
-  double dredw[kCWarps];  // per-warp sums of the clipped d_E (winsorised min-max) or of s_E (MAD scaling)
-  unsigned wsum[kCWarps];
-  alignas(16) int wscan[kCWarps][4];  // per-warp counts above / equal to the threshold, and of lower ranks' keys
+  double dred[Shape<kSh>::kWarps];   // per-warp sums of S_imp (value-norm importance)
+  double dredw[Shape<kSh>::kWarps];  // per-warp sums of the clipped d_E (winsorised) or of s_E (MAD scaling)
+  unsigned wsum[Shape<kSh>::kWarps];
+  // per-warp counts above / equal to the threshold, and of lower ranks' keys
+  alignas(16) int wscan[Shape<kSh>::kWarps][4];
   int shi[4];
   unsigned lcount;        // keys this CTA has put on the list
 };
@@ -198,7 +203,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
       const float* Su = f.S + (size_t)u * Tv;
 #pragma unroll 8
       for (int j = 0; j < kJ; ++j) {
-        const int i = lo + kCThreads * j + tid;
+        const int i = lo + Shape<kSh>::kThreads * j + tid;
         if (i < Tv) sm.raw()[pad_idx(i - lo + kHalo)] = ld(Su + i);
       }
       __syncthreads();
@@ -221,7 +226,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
       peers_started();
       if (tid < C) {
         unsigned a0 = __float_as_uint(sm.red[0][0]), a1 = __float_as_uint(sm.red[0][1]);
-        for (int w = 1; w < kCWarps; ++w) {
+        for (int w = 1; w < Shape<kSh>::kWarps; ++w) {
           a0 = min(a0, __float_as_uint(sm.red[w][0]));
           a1 = max(a1, __float_as_uint(sm.red[w][1]));
         }
@@ -251,7 +256,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
     auto load_batch = [&](int b0) {
 #pragma unroll
       for (int j = 0; j < kBatch; ++j) {
-        const int i = lo + 4 * (kCThreads * (b0 + j) + tid);
+        const int i = lo + 4 * (Shape<kSh>::kThreads * (b0 + j) + tid);
         ea[j] = ca[j] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (i + 3 < Tv) {
           ea[j] = ld4(dEu + i);
@@ -267,7 +272,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
     //    d_E, sums of cosines and of raw votes over the candidates); meanwhile
     //    the CTA's raw votes with the pooling halo and the edge values
     float v6[6] = {0.f, INFINITY, -INFINITY, 0.f, 0.f, 0.f};
-    for (int ch = tid; ch < f.nchunks; ch += kCThreads) {
+    for (int ch = tid; ch < f.nchunks; ch += Shape<kSh>::kThreads) {
       const float* p = f.p2part + ((size_t)u * f.nchunks + ch) * kP2Stride;
       v6[0] += ld(p + P2_SUM_DE_ALL);
       v6[1] = fminf(v6[1], ld(p + P2_MIN_DE));
@@ -281,7 +286,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
         // the whole halo of kHalo each side in 16-byte loads (kHalo and lo are
         // multiples of four, so each group of four lies inside [0, Tv) or
         // outside it entirely except at the ragged end)
-        for (int q = 4 * tid; q < kCap + 2 * kHalo; q += 4 * kCThreads) {
+        for (int q = 4 * tid; q < kCap + 2 * kHalo; q += 4 * Shape<kSh>::kThreads) {
           const int j = lo - kHalo + q;
           float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
           if (j >= 0 && j + 3 < Tv) {
@@ -297,7 +302,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
           sm.raw()[pad_idx(q + 3)] = v.w;
         }
       } else {
-        for (int q = kHalo - hpool + tid; q < kHalo + kCap + hpool; q += kCThreads) {
+        for (int q = kHalo - hpool + tid; q < kHalo + kCap + hpool; q += Shape<kSh>::kThreads) {
           const int j = lo - kHalo + q;
           sm.raw()[pad_idx(q)] = (j >= 0 && j < Tv) ? ld(raw + j) : 0.f;
         }
@@ -357,7 +362,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
     // every thread takes the extrema of d_E from the warps' partials
     float mnE = sm.red[0][1], wmax = sm.red[0][2];
 #pragma unroll
-    for (int w = 1; w < kCWarps; ++w) {
+    for (int w = 1; w < Shape<kSh>::kWarps; ++w) {
       mnE = fminf(mnE, sm.red[w][1]);
       wmax = fmaxf(wmax, sm.red[w][2]);
     }
@@ -402,7 +407,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
       const float* vnu = f.vnorm + (size_t)u * Tv;
   #pragma unroll 8
       for (int j = 0; j < kJ; ++j) {
-        const int i = lo + kCThreads * j + tid;
+        const int i = lo + Shape<kSh>::kThreads * j + tid;
         if (i < Tv) sm.raw()[pad_idx(i - lo + kHalo)] = ld(vnu + i);
       }
       __syncthreads();
@@ -429,7 +434,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
       // weighs two terms of order one: its rounding stays at the level of the
       // scores' own)
       float s_all = sm.red[0][0];
-      for (int w = 1; w < kCWarps; ++w) s_all += sm.red[w][0];
+      for (int w = 1; w < Shape<kSh>::kWarps; ++w) s_all += sm.red[w][0];
       const float D_E = __fdiv_rn(s_all, (float)f.N);
       const float tau = f.tau > 0.f ? f.tau : sqrtf((float)kD);
       const float r_E = 2.f - 2.f / (1.f + expf(-D_E / tau));
@@ -442,7 +447,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
       // means, in double and scaled by Tv: sum_i S_imp(i) = (1/kp) sum_j
       // raw(j) cnt(j), where cnt(j) = kp except within kp/2 of either end
       float s_raw = sm.red[0][5];
-      for (int w = 1; w < kCWarps; ++w) s_raw += sm.red[w][5];
+      for (int w = 1; w < Shape<kSh>::kWarps; ++w) s_raw += sm.red[w][5];
       // (the edge terms as a sum of two floats, exact to 2^-46: a loop in
       // double takes 1.5 us here)
       const int h = hpool;
@@ -465,7 +470,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
     } else if (tid == 96) {
       // mean(Sbar) is affine in the means of d_E and of the cosine (as finalize_unit)
       float s_de = sm.red[0][3], s_c = sm.red[0][4];
-      for (int w = 1; w < kCWarps; ++w) {
+      for (int w = 1; w < Shape<kSh>::kWarps; ++w) {
         s_de += sm.red[w][3];
         s_c += sm.red[w][4];
       }
@@ -508,7 +513,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
         if (!kEarly) load_batch(b0);
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
-          const int i = lo + 4 * (kCThreads * (b0 + j) + tid);
+          const int i = lo + 4 * (Shape<kSh>::kThreads * (b0 + j) + tid);
           if (i + 3 < Tv) {
             sweep1(i, ea[j].x, ca[j].x);
             sweep1(i + 1, ea[j].y, ca[j].y);
@@ -519,7 +524,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
       }
     }
 #pragma unroll 8
-    for (int i = tail + tid; i < hi; i += kCThreads) sweep1(i, ld(dEu + i), ld(cvu + i));
+    for (int i = tail + tid; i < hi; i += Shape<kSh>::kThreads) sweep1(i, ld(dEu + i), ld(cvu + i));
     if (wins || madv) {
       double wsum = (double)wsumf;
   #pragma unroll
@@ -537,19 +542,19 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
     if (tid < C) {  // one thread a peer
       float4 a = sm.red4[0];
 #pragma unroll
-      for (int w = 1; w < kCWarps; ++w) {
+      for (int w = 1; w < Shape<kSh>::kWarps; ++w) {
         const float4 b = sm.red4[w];
         a = make_float4(fminf(a.x, b.x), fmaxf(a.y, b.y), fminf(a.z, b.z), fmaxf(a.w, b.w));
       }
       *cl.map_shared_rank(&sm.ext_all[rank], tid) = a;
       if (kVar && f.vnorm != nullptr) {
         double cs = 0.0;
-        for (int w = 0; w < kCWarps; ++w) cs += sm.dred[w];
+        for (int w = 0; w < Shape<kSh>::kWarps; ++w) cs += sm.dred[w];
         *cl.map_shared_rank(&sm.simp_all[rank], tid) = cs;
       }
       if (wins || madv) {
         double cs = 0.0;
-        for (int w = 0; w < kCWarps; ++w) cs += sm.dredw[w];
+        for (int w = 0; w < Shape<kSh>::kWarps; ++w) cs += sm.dredw[w];
         *cl.map_shared_rank(&sm.wsum_all[rank], tid) = cs;
       }
     }
@@ -641,7 +646,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
       if (vec4) {
   #pragma unroll 4
         for (int j = 0; j < kJ / 4; ++j) {
-          const int i = lo + 4 * (kCThreads * j + tid);
+          const int i = lo + 4 * (Shape<kSh>::kThreads * j + tid);
           const int q = i - lo + kHalo;
           if (i + 3 < Tv) {
             *reinterpret_cast<float4*>(Sg + i) =
@@ -653,7 +658,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
       } else {
   #pragma unroll 8
         for (int j = 0; j < kJ; ++j) {
-          const int i = lo + kCThreads * j + tid;
+          const int i = lo + Shape<kSh>::kThreads * j + tid;
           if (i < Tv) Sg[i] = sm.raw()[pad_idx(i - lo + kHalo)];
         }
       }
@@ -665,7 +670,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
     unsigned thr = 0u;
     int rem = k;               // keys still to take from the range [klo, khi]
     int gt_low = 0, eq_low = 0;  // this thread's share of the lower ranks' keys above / equal to thr
-    constexpr int kBins = Shape<kSh>::kBins, kPer = kBins / kCThreads;  // ranges a thread sums
+    constexpr int kBins = Shape<kSh>::kBins, kPer = kBins / Shape<kSh>::kThreads;  // ranges a thread sums
     if (k > 0) {
       int pass = 0;
       for (bool first = true;; first = false) {
@@ -732,7 +737,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
         if (lane == 0) sm.wsum[warp] = suf;
         __syncthreads();
 #pragma unroll
-        for (int w = 0; w < kCWarps; ++w)
+        for (int w = 0; w < Shape<kSh>::kWarps; ++w)
           if (w > warp) suf += sm.wsum[w];
         if (suf >= (unsigned)rem && suf - tot < (unsigned)rem) {
           unsigned above = suf - tot;
@@ -785,14 +790,14 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
           for (int c = 0; c < kJ; ++c)
             if (c < nv && key[c] >= klo && key[c] <= khi) sm.hist[atomicAdd(&sm.lcount, 1u)] = key[c];
           __syncthreads();
-          for (unsigned t = tid; t < sm.lcount; t += kCThreads)
+          for (unsigned t = tid; t < sm.lcount; t += Shape<kSh>::kThreads)
             for (int r = 0; r < C; ++r) *cl.map_shared_rank(&sm.list[before + t], r) = sm.hist[t];
           if (tid < 3) sm.list[min(cnt + tid, kList + 2)] = 0u;  // the last group of four: below every key
           unit_sync(C);
           // 2^sp threads a key, each comparing it with every 2^sp-th group of four
           const int sp = cnt <= 32 ? 3 : (cnt <= 64 ? 2 : (cnt <= 128 ? 1 : 0));
           const int seg = tid & ((1 << sp) - 1);
-          for (int t0 = 0; t0 < cnt; t0 += kCThreads >> sp) {
+          for (int t0 = 0; t0 < cnt; t0 += Shape<kSh>::kThreads >> sp) {
             const int t = t0 + (tid >> sp);
             const unsigned x = sm.list[min(t, cnt - 1)];
             int g = 0, e = 0;
@@ -814,7 +819,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
           __syncthreads();
           thr = sm.wsum[0];
           rem = (int)sm.wsum[1];
-          for (int t = tid; t < before; t += kCThreads) {
+          for (int t = tid; t < before; t += Shape<kSh>::kThreads) {
             gt_low += sm.list[t] > thr;
             eq_low += sm.list[t] == thr;
           }
@@ -859,7 +864,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
     __syncthreads();
     int gt_excl = gi - n_gt, eq_excl = ei - n_eq, pos = 0, eq_before = 0;
 #pragma unroll
-    for (int w = 0; w < kCWarps; ++w) {
+    for (int w = 0; w < Shape<kSh>::kWarps; ++w) {
       const int4 v = *reinterpret_cast<const int4*>(sm.wscan[w]);
       if (w < warp) {
         gt_excl += v.x;
@@ -883,14 +888,14 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
     if (keep_all) {
       // B >= N: every row in order; rank r writes its candidates, the last rank the window
       const int hi = min(Tv, lo + kCap);
-      for (int i = lo + tid; i < hi; i += kCThreads) out[i] = i;
+      for (int i = lo + tid; i < hi; i += Shape<kSh>::kThreads) out[i] = i;
       if (rank == C - 1)
-        for (int j = tid; j < f.W; j += kCThreads) out[Tv + j] = Tv + j;
+        for (int j = tid; j < f.W; j += Shape<kSh>::kThreads) out[Tv + j] = Tv + j;
     } else if (rank == C - 1) {
-      for (int j = tid; j < f.W; j += kCThreads) out[k + j] = Tv + j;
+      for (int j = tid; j < f.W; j += Shape<kSh>::kThreads) out[k + j] = Tv + j;
     }
     if (rank == C - 1)  // slots past this unit's budget (per-layer budgets) hold -1
-      for (int r = (keep_all ? f.N : budget) + tid; r < f.n_keep; r += kCThreads) out[r] = -1;
+      for (int r = (keep_all ? f.N : budget) + tid; r < f.n_keep; r += Shape<kSh>::kThreads) out[r] = -1;
   }
   // No CTA touches a peer's shared memory after the last cluster barrier it
   // passed (every exchange is a store made before that barrier), so the
