@@ -25,9 +25,24 @@ __global__ void __launch_bounds__(Shape<kSh>::kThreads, Shape<kSh>::kMinCtas) fi
   cluster_unit<kMode, kSh, kVar, false>(f, sm, cl, blockIdx.x / C, (int)cl.block_rank(), C);
 }
 
+// Shared memory a CTA asks for: what it uses, or so much that an SM takes two
+// (spread 1) or one (spread 2).  A cluster is placed as soon as one GPC has
+// room for it, while the streaming pass still runs on the other SMs; with what
+// it uses alone its CTAs then share the two or four SMs that are free first, and
+// each runs at a fraction of its speed.  One layer, us a call as used / two /
+// one an SM: 4 heads x 32768 keys (16 CTAs each) 59.5 / 53.3 / 50.0, 8 x 65536
+// (8 CTAs of 32 candidates a thread) 112 / 99.5 / 90.9, 8 x 8192 38.1 / 35.8 /
+// 35.8; but 8 x 131072, whose clusters of 16 are not all resident at one an SM,
+// 149 / 142 / 158.
+template <int kSh>
+constexpr int smem_bytes(int spread) {
+  const int used = (int)sizeof(ClusterSmem<kSh>), wide = spread == 2 ? 200 * 1024 : (spread == 1 ? 110 * 1024 : 0);
+  return used > wide ? used : wide;
+}
+
 template <int kSh>
 cudaError_t set_attrs(bool nonportable) {
-  const int bytes = (int)sizeof(ClusterSmem<kSh>);
+  const int bytes = smem_bytes<kSh>(2);
   const void* kernels[5] = {(const void*)finalize_cluster_kernel<0, kSh, false>,
                             (const void*)finalize_cluster_kernel<1, kSh, false>,
                             (const void*)finalize_cluster_kernel<0, kSh, true>,
@@ -42,11 +57,11 @@ cudaError_t set_attrs(bool nonportable) {
 }
 
 template <int kSh>
-cudaError_t launch_shape(const FinalArgs& f, int U, int C, bool select_only, cudaStream_t s) {
+cudaError_t launch_shape(const FinalArgs& f, int U, int C, int spread, bool select_only, cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(U * C), 1, 1);
   cfg.blockDim = dim3(Shape<kSh>::kThreads, 1, 1);
-  cfg.dynamicSmemBytes = sizeof(ClusterSmem<kSh>);
+  cfg.dynamicSmemBytes = smem_bytes<kSh>(spread);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -69,20 +84,21 @@ cudaError_t launch_shape(const FinalArgs& f, int U, int C, bool select_only, cud
 // Per device: the attributes set, and whether clusters of 16 CTAs of the
 // longest shape can be resident (cudaOccupancyMaxActiveClusters > 0).
 std::atomic<int> g_setup[64];  // 0 = not yet, 1 = set, clusters of 16 unavailable, 2 = set and available
-// Clusters of C CTAs of shapes 0-3 resident at once plus one, at [shape][C - 1]; 0 = not asked yet.
-std::atomic<int> g_fit[64][4][16];
+// Clusters of C CTAs of shapes 0-3 resident at once plus one, at [shape][spread][C - 1]; 0 = not asked yet.
+std::atomic<int> g_fit[64][4][3][16];
+std::atomic<int> g_sms[64];  // SMs, set before g_setup
 
 // Clusters of C CTAs that the current device holds at once (the occupancy
 // query's answer, asked once; a racing thread asks again).
 template <int kSh>
-int clusters_fit(int dev, int C) {
-  int n = g_fit[dev][kSh][C - 1].load();
+int clusters_fit(int dev, int C, int spread) {
+  int n = g_fit[dev][kSh][spread][C - 1].load();
   if (n > 0) return n - 1;
   n = 0;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)C * 1024u, 1, 1);
   cfg.blockDim = dim3(Shape<kSh>::kThreads, 1, 1);
-  cfg.dynamicSmemBytes = sizeof(ClusterSmem<kSh>);
+  cfg.dynamicSmemBytes = smem_bytes<kSh>(spread);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)C;
@@ -94,14 +110,17 @@ int clusters_fit(int dev, int C) {
     cudaGetLastError();  // an unavailable configuration leaves no error behind
     n = 0;
   }
-  g_fit[dev][kSh][C - 1].store(n + 1);
+  g_fit[dev][kSh][spread][C - 1].store(n + 1);
   return n;
 }
 
-int clusters_fit(int dev, int sh, int C) {
-  return sh == 0 ? clusters_fit<0>(dev, C) : sh == 1 ? clusters_fit<1>(dev, C)
-                                         : sh == 2   ? clusters_fit<2>(dev, C)
-                                                     : clusters_fit<3>(dev, C);
+int clusters_fit(int dev, int sh, int C, int spread) {
+  switch (sh) {
+    case 0: return clusters_fit<0>(dev, C, spread);
+    case 1: return clusters_fit<1>(dev, C, spread);
+    case 2: return clusters_fit<2>(dev, C, spread);
+  }
+  return clusters_fit<3>(dev, C, spread);
 }
 
 int device_setup() {
@@ -112,8 +131,11 @@ int device_setup() {
   if (set_attrs<0>(false) != cudaSuccess || set_attrs<1>(false) != cudaSuccess || set_attrs<2>(false) != cudaSuccess ||
       set_attrs<3>(false) != cudaSuccess || set_attrs<5>(false) != cudaSuccess)
     return -1;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return -1;
+  g_sms[dev].store(sms);
   const bool wide = set_attrs<0>(true) == cudaSuccess && set_attrs<3>(true) == cudaSuccess;
-  st = wide && clusters_fit<3>(dev, 16) > 0 ? 2 : 1;
+  st = wide && clusters_fit<3>(dev, 16, 0) > 0 ? 2 : 1;
   cudaGetLastError();  // an unavailable configuration leaves no error behind
   g_setup[dev].store(st);
   return st;
@@ -123,9 +145,10 @@ int device_setup() {
 // them.  The fewest candidates a thread whose clusters are all resident at once
 // (one layer of 4 heads x 32768 keys: 16 CTAs of 8 a thread 15 us, 4 of 32 a
 // thread 25 us; 28 layers x 4 heads of that length: 3 waves of the former, one
-// of the latter).  Failing that (many units) clusters of at most four: of
-// 128-thread CTAs up to 8192 candidates, seven to an SM (32 x 32 heads of 2048
-// keys: 21 us against 27 in CTAs of 256 threads, 608 at once; 20 x 32 of 6000
+// of the latter), and where they are at most one an SM in number, spread so
+// (smem_bytes; two an SM asked of 224 CTAs, 28 x 4 heads of 14500 keys, cost 2
+// us).  Failing that (many units) clusters of at most four: of 128-thread CTAs
+// up to 8192 candidates, seven to an SM (32 x 32 heads of 2048 keys: 21 us against 27 in CTAs of 256 threads, 608 at once; 20 x 32 of 6000
 // keys 42 against 53), else the fewest candidates a thread.  The 128-thread
 // CTAs in clusters of more than four, resident at once, lost to 32 candidates a
 // thread (28 x 4 heads of 16411 keys, nine CTAs each: 234 against 218 us a
@@ -133,14 +156,18 @@ int device_setup() {
 // alone, 112 clusters of four at three CTAs an SM would fit, but the SMs of a
 // GPC hold whole clusters only (28 x 4 heads of 14500 keys: 202 us a call in
 // two waves of those, 194 in one of 32 candidates a thread).
-void pick_shape(int Tv, long long U, int dev, bool long_ok, int& sh, int& C) {
+void pick_shape(int Tv, long long U, int dev, bool long_ok, int& sh, int& C, int& spread) {
+  spread = 0;
   const int t = Tv > 0 ? Tv : 1;
   const int cap[4] = {Shape<0>::kCap, Shape<1>::kCap, Shape<2>::kCap, Shape<3>::kCap};
   const int most[4] = {long_ok ? Shape<0>::kMaxCluster : 8, Shape<1>::kMaxCluster, Shape<2>::kMaxCluster,
                        long_ok ? Shape<3>::kMaxCluster : 8};
   for (sh = 0; sh < 4; ++sh) {
     C = (t + cap[sh] - 1) / cap[sh];
-    if (C <= most[sh] && U <= clusters_fit(dev, sh, C)) return;
+    if (C <= most[sh] && U <= clusters_fit(dev, sh, C, 0)) {
+      while (U * C <= g_sms[dev].load() && spread < 2 && U <= clusters_fit(dev, sh, C, spread + 1)) ++spread;
+      return;
+    }
   }
   sh = 5;
   C = (t + Shape<5>::kCap - 1) / Shape<5>::kCap;
@@ -163,22 +190,22 @@ int current_device() {
 bool cluster_finalize_fits(int Tv) {
   const int st = device_setup();
   if (st < 0) return false;
-  int sh, C;
-  pick_shape(Tv, 1, current_device(), st == 2, sh, C);
+  int sh, C, spread;
+  pick_shape(Tv, 1, current_device(), st == 2, sh, C, spread);
   return sh >= 0;
 }
 
 cudaError_t launch_finalize_cluster(const FinalArgs& f, int U, bool select_only, cudaStream_t s) {
   const int st = device_setup();
   if (st < 0) return cudaErrorUnknown;
-  int sh, C;
-  pick_shape(f.Tv, U, current_device(), st == 2, sh, C);
+  int sh, C, spread;
+  pick_shape(f.Tv, U, current_device(), st == 2, sh, C, spread);
   switch (sh) {
-    case 0: return launch_shape<0>(f, U, C, select_only, s);
-    case 1: return launch_shape<1>(f, U, C, select_only, s);
-    case 2: return launch_shape<2>(f, U, C, select_only, s);
-    case 3: return launch_shape<3>(f, U, C, select_only, s);
-    case 5: return launch_shape<5>(f, U, C, select_only, s);
+    case 0: return launch_shape<0>(f, U, C, spread, select_only, s);
+    case 1: return launch_shape<1>(f, U, C, spread, select_only, s);
+    case 2: return launch_shape<2>(f, U, C, spread, select_only, s);
+    case 3: return launch_shape<3>(f, U, C, spread, select_only, s);
+    case 5: return launch_shape<5>(f, U, C, spread, select_only, s);
   }
   return cudaErrorNotSupported;
 }
