@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
     const int t = threadIdx.x - 128;
     uint32_t qpar = 0u;    // per slot: parity of the next qfull phase (completed by P1 and P2 items)
     uint32_t tcnt = 0;     // tiles of the items so far
-    bool after_p2 = false;
+    uint32_t guarded = 0;  // tiles before this one may follow a pass-2 tile in their stage
     uint32_t sphase = 0u;  // of statbar, the bounded barrier among the four warps
     auto stat_sync = [&]() -> bool {
       __syncwarp();
@@ -547,21 +547,23 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
       if (type == kExit) break;
       const uint32_t ntiles = (uint32_t)d.ntiles;
       if (C::kStatNorms && type == kP1) {
-        // (a stage's phase may only be waited for once the one before it is
-        // complete: after pass-2 tiles, which these warps do not wait for,
-        // the ring's last tiles first; they are all issued by now)
-        if (after_p2)
-          for (uint32_t q = tcnt > (uint32_t)kS ? tcnt - kS : 0u; q < tcnt && ok; ++q)
-            ok = wait_warp(&s.full[q % kS], (q / kS) & 1u, a, 24u);
-        after_p2 = false;
+        // A landed phase may only be waited for once the one before it is
+        // complete.  The stage's last tile may be one of pass 2, which these
+        // warps neither wait for nor release; its own landed phase may long
+        // have been overtaken (the producer runs ahead while records are
+        // folded below), but its release cannot: the tile that follows in the
+        // stage, this one, is not released without these warps, and with this
+        // item published the last tile before it in the stage is issued, the
+        // one before that released.
+        for (uint32_t q = tcnt; q < min(guarded, tcnt + ntiles) && ok; ++q)
+          ok = wait_warp(&s.empty[q % kS], ((q / kS) & 1u) ^ 1u, a, 24u);
         for (uint32_t q = tcnt; q < tcnt + ntiles && ok; ++q)
           if ((ok = wait_warp(&s.full[q % kS], (q / kS) & 1u, a, 25u)))
             key_work(q % kS, t, d.i0 + (int)(q - tcnt) * kTile + t);
         if (!ok) break;
-      } else if (type == kP2) {
-        after_p2 = true;
       }
       tcnt += ntiles;
+      if (type == kP2) guarded = tcnt + kS;
       if (type == kP2) {
         int c0, nrec;
         unit_slices(a, u, c0, nrec);

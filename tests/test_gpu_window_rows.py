@@ -49,3 +49,21 @@ def test_128_rows_in_one_launch(group, window):
     # the odd last tile with keys that not every row sees
     run_and_compare(small_workload(33001, h_kv=8, group=group, window=window, budget=3300, dtype="bf16", seed=6),
                     units=[(0, 0), (0, 7)])
+
+
+# waves of few heads past 64 window rows, where the warps that fold the
+# statistics also compute pass 1's norms: their wait for a key tile that follows
+# tiles of pass 2 in the ring (slices of one to three tiles, and of more tiles
+# than the ring has stages)
+@pytest.mark.parametrize("n,wave,lag", [(5000, 1, 1), (5000, 1, 2), (5000, 2, 1), (5000, 5, 1), (19500, 1, 1),
+                                        (19500, 5, 1), (40001, 3, 1)], ids=lambda v: str(v))
+def test_schedules_of_112_rows(n, wave, lag):
+    run_and_compare(small_workload(n, h_kv=2, group=7, window=16, budget=500, dtype="bf16", n_layers=3, seed=8,
+                                   clustered=True),
+                    units=[(0, 0), (1, 1), (2, 1)], sched_wave=wave, sched_lag=lag, timeout_us=200000)
+
+
+@pytest.mark.parametrize("wave,lag", [(1, 1), (2, 1), (5, 1), (3, 2)], ids=lambda v: str(v))
+def test_schedules_of_128_rows_in_one_launch(wave, lag):
+    run_and_compare(small_workload(33001, h_kv=8, group=8, window=16, budget=3300, dtype="bf16", seed=6),
+                    units=[(0, 0), (0, 7)], sched_wave=wave, sched_lag=lag, timeout_us=200000)
