@@ -279,12 +279,11 @@ static ecokv_status run_tc_group(const ecokv_params& p, const Layout& L, const v
 
 // Short units: score (and, with f.idx, select) by one cluster per unit in one
 // launch.  CTAs a unit takes, 0 where the call goes another way: the variants
-// that need another launch between the passes and the finalisation, a streaming
-// schedule asked for, and the injected stall, which lives in the persistent
-// kernel.
+// that need another launch between the passes and the finalisation, and a
+// streaming schedule asked for.
 static int short_ctas(const ecokv_params& p, ecokv_dtype dt) {
   if (!use_tensor_path(p, dt) || p.sched_wave != 0 || p.sched_lag != 0) return 0;
-  if (p.flags & (ECOKV_FLAG_VNORM_IMP | ECOKV_FLAG_WINSOR_1 | ECOKV_FLAG_WINSOR_5 | ECOKV_FLAG_MAD | ECOKV_FLAG_TEST_STALL))
+  if (p.flags & (ECOKV_FLAG_VNORM_IMP | ECOKV_FLAG_WINSOR_1 | ECOKV_FLAG_WINSOR_5 | ECOKV_FLAG_MAD))
     return 0;
   const int C =
       short_cluster((p.h_q / p.h_kv) * p.window, (p.n + 127) / 128, (long long)p.n_layers * p.h_kv, num_sms());
@@ -306,6 +305,7 @@ static ecokv_status run_short(const ecokv_params& p, const Layout& L, const void
   a.kbar_n = kbar_count(p, L);
   a.q_rows = p.n_layers * p.h_q * p.window;
   a.ustat_stride = L.ustat_stride;
+  a.stall_unit = (p.flags & ECOKV_FLAG_TEST_STALL) ? 0 : -1;
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)p.d));
   a.timeout_ns = wait_limit_ns(p);
   a.Q = Q;

@@ -59,6 +59,7 @@ struct ShortArgs {
   int kbar_n;                       // keys 0 .. kbar_n - 1 form the centroid
   int q_rows;                       // rows of the window-query tensor
   int ustat_stride;
+  int stall_unit;                   // fault injection: this unit's statistics never complete (-1: none)
   float scale_log2;
   unsigned long long timeout_ns;    // limit of every bounded wait (global timer)
   const void* Q;

@@ -33,7 +33,9 @@
 //      grid: by the CTAs that keep the rows it took 2 us longer.)
 // Every wait on an mbarrier is bounded; a wait that runs out records
 // ECOKV_ERR_TIMEOUT, and the CTA goes through the remaining barriers without
-// waiting for anything else (outputs unspecified).
+// waiting for anything else but the end of its own copies and MMAs.  The CTAs
+// of a cluster tell each other: when one gave up none of them finalises (the
+// unit's outputs are unspecified).
 
 #include <cuda.h>
 
@@ -78,6 +80,7 @@ struct __align__(1024) ShortSmem {
   alignas(16) float ust[2 * kD + 4 + RP];   // kbar, mu, their squared norms (two halves each), negated log2-sum-exp
   float red6[kWarps][8];
   uint64_t full[kShortTiles], tfull[kShortTiles], qfull, sigma, stat;
+  uint32_t gave_up[kShortCtas];             // written by the peers: whether a wait of theirs ran out
   uint32_t tmem_base;
 };
 static_assert(offsetof(ShortSmem<8>, ktile) == 0, "the key tiles come first");
@@ -96,6 +99,14 @@ __device__ __forceinline__ bool wait_limit(uint64_t* bar, uint32_t parity, const
       return false;
     }
   return true;
+}
+
+// The same for what this CTA has itself set in motion, after a wait has run out:
+// nothing is recorded.
+__device__ void drain(uint64_t* bar, const ShortArgs& a) {
+  const unsigned long long t0 = now_ns();
+  while (!mbar_try_wait(bar, 0u) && now_ns() - t0 < a.timeout_ns) {
+  }
 }
 
 template <int RP, bool kSelect>
@@ -163,6 +174,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   };
 
   // 1. logits MMAs as the tiles land
+  int logits_issued = 0;  // by warp 0: tiles
+  bool sums_issued = false, stats_issued = false;
   if (warp == 0) {
     constexpr uint32_t idesc = idesc_bf16(128, SC::kNQ, false, false);
     const uint64_t kd0 = smem_desc(smem_u32(s.ktile[0]), 16, 1024, 2);
@@ -179,6 +192,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    qd + (uint64_t)((k8 >> 2) * (SC::kNQ * 8) + (k8 & 3) * 2), idesc, k8 > 0 ? 1u : 0u);
         mma_commit(&s.tfull[t]);
       }
+      if (ok) logits_issued = t + 1;
       __syncwarp();
     }
   }
@@ -199,7 +213,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   fence_proxy_async_smem();
   __syncthreads();
   // sums of k and k/||k|| over the CTA's keys
-  if (warp == 0 && ok && elect_one()) {
+  sums_issued = warp == 0 && ok;
+  if (sums_issued && elect_one()) {
     tc_fence_after();
     constexpr uint32_t idesc = idesc_bf16(128, 16, true, false);
     const uint64_t kd0 = smem_desc(smem_u32(s.ktile[0]), kTileBytes / 2, 1024, 2);
@@ -304,7 +319,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   fence_proxy_async_smem();
   __syncthreads();
   // 3. k . kbar and k . mu of every key
-  if (warp == 0 && ok && elect_one()) {
+  // (the injected stall: the first CTA of one unit never has them)
+  stats_issued = warp == 0 && ok && !(u == a.stall_unit && rank == 0);
+  if (stats_issued && elect_one()) {
     constexpr uint32_t idesc = idesc_bf16(128, 16, false, false);
     const uint64_t kd0 = smem_desc(smem_u32(s.ktile[0]), 16, 1024, 2);
     const uint64_t sd = smem_desc(smem_u32(s.srow[0]), 16, 1024, 2);
@@ -383,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     s.red6[warp][P2_SUM_RAW] = s_raw;
   }
   tc_fence_before();
-  __syncthreads();
+  const bool gave_up = __syncthreads_or(ok ? 0 : 1) != 0;
   if (tid < 6) {
     float acc = s.red6[0][tid];
 #pragma unroll
@@ -394,19 +411,27 @@ __global__ void __launch_bounds__(kThreads, 1)
     a.p2part[((size_t)u * C + rank) * kP2Stride + tid] = acc;
   }
   if (tid == 32 && rank == 0) a.ustat[(size_t)u * a.ustat_stride + ustat_musq()] = s.ust[2 * kD + 2] + s.ust[2 * kD + 3];
-  if (!ok) {
-    // a wait ran out: let this CTA's copies and MMAs in flight end (bounded)
-    // before its memory changes hands
-    for (int t = 0; t < nt; ++t) wait_limit(&s.full[t], 0u, a, 46u);
-    wait_limit(&s.qfull, 0u, a, 46u);
+  if (gave_up) {
+    // a wait ran out: the copies and MMAs in flight end (bounded) before this
+    // CTA's memory changes hands
+    for (int t = 0; t < logits_issued; ++t) drain(&s.tfull[t], a);
+    if (sums_issued) drain(&s.sigma, a);
+    if (stats_issued) drain(&s.stat, a);
+    for (int t = 0; t < nt; ++t) drain(&s.full[t], a);
+    drain(&s.qfull, a);
+    __syncthreads();
   }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
+  if (tid < C) *cl.map_shared_rank(&s.gave_up[rank], tid) = gave_up ? 1u : 0u;
   // 4. what every CTA of the cluster has written is read by all of them
   __threadfence();
   unit_sync(C);
+  // a CTA whose keys never came has nothing to finalise, and its peers would
+  // take its counts for theirs: all of them stop here
+  if (__any_sync(0xffffffffu, lane < C && s.gave_up[lane] != 0u)) return;
   cluster_unit<kSelect ? 1 : 0, 4, false, true>(f, *reinterpret_cast<ClusterSmem<4>*>(&s), cl, u, rank, C);
 }
 

@@ -1,7 +1,9 @@
 """Bounded device-side waits, made to run out on purpose without faulting the
 GPU: with ECOKV_FLAG_TEST_STALL the statistics of the first unit never
 complete (the streaming kernel expects one more pass-1 arrival than there are
-pass-1 items), so the wait of its pass 2 gives up after timeout_us.  The call
+pass-1 items; the short-unit kernel, which takes this shape unless a schedule
+is asked for, leaves out the product of one CTA's keys with the statistics), so
+the wait of its pass 2 gives up after timeout_us.  The call
 must report ECOKV_ERR_TIMEOUT through ecokv_device_status, return well before
 the default 2 s limit, and leave the context and the workspace usable: the
 next call on the same workspace is bit for bit the call on a fresh one, and
@@ -25,12 +27,13 @@ def params_of(w, **kw):
                          budget=w.budget, pool_kernel=w.pool_kernel, **kw)
 
 
-def test_stalled_statistics_time_out_and_the_workspace_recovers():
+@pytest.mark.parametrize("sched_wave", [0, 4], ids=["short_units", "streaming"])
+def test_stalled_statistics_time_out_and_the_workspace_recovers(sched_wave):
     w = small_workload(3000, h_kv=2, group=4, window=8, budget=300, dtype="bf16", n_layers=2, clustered=True)
     K, V, Q = make_inputs(w)
     Kd, Vd, Qd = K.to(DEV), V.to(DEV), Q.to(DEV)
-    p_stall = params_of(w, flags=E.ECOKV_FLAG_TEST_STALL, timeout_us=20000)
-    p = params_of(w)
+    p_stall = params_of(w, flags=E.ECOKV_FLAG_TEST_STALL, timeout_us=20000, sched_wave=sched_wave)
+    p = params_of(w, sched_wave=sched_wave)
     assert E.ecokv_workspace_size(p_stall) == E.ecokv_workspace_size(p)
     ws = E.alloc_workspace(p, DEV)
     torch.cuda.synchronize()
@@ -60,6 +63,25 @@ def test_stalled_statistics_time_out_and_the_workspace_recovers():
         check_selection(idx[l, h].cpu().numpy(), r, op, TOL["bf16"], what)
         check_rows(Kd[l, h], idx[l, h], Ko[l, h], what)
         check_rows(Vd[l, h], idx[l, h], Vo[l, h], what)
+
+
+def test_a_unit_that_gave_up_is_not_finalised():
+    """Short units: where one CTA of a cluster gave up none of them goes on to
+    the scores (their memory may still be the target of copies, and the counts
+    they exchange would be those of no selection); the other units' results
+    are those of an undisturbed call."""
+    w = small_workload(3000, h_kv=2, group=4, window=8, budget=300, dtype="bf16", n_layers=2, clustered=True)
+    K, V, Q = (t.to(DEV) for t in make_inputs(w))
+    p_stall = params_of(w, flags=E.ECOKV_FLAG_TEST_STALL, timeout_us=20000)
+    want = E.evict(params_of(w), K, V, Q, want_scores=True)
+    ws = E.alloc_workspace(p_stall, DEV)
+    idx, Ko, Vo, S, lam = (torch.full_like(t, -7) for t in want)
+    assert E.ecokv_evict(p_stall, E.dtype_code(K), K, V, Q, idx, Ko, Vo, S, lam, ws, ws.numel()) == 0
+    assert E.ecokv_device_status(ws) == E.ECOKV_ERR_TIMEOUT
+    for t in (S, lam, idx):
+        assert bool((t[0, 0] == -7).all())
+    for got, ref in zip((idx, Ko, Vo, S, lam), want):
+        assert torch.equal(got[0, 1], ref[0, 1]) and torch.equal(got[1], ref[1])
 
 
 def test_stall_flag_needs_the_tensor_core_path():
