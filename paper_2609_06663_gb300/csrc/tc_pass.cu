@@ -193,14 +193,6 @@ __device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, const 
   return __all_sync(0xffffffffu, wait_bar(bar, parity, a, where)) != 0;
 }
 
-// Wait for an mbarrier phase without regard to the abort flag, bounded: the
-// drain of copies in flight before a CTA leaves.
-__device__ void drain_bar(uint64_t* bar, uint32_t parity, const TcArgs& a) {
-  const unsigned long long t0 = now_ns();
-  while (!mbar_try_wait(bar, parity) && now_ns() - t0 < a.timeout_ns) {
-  }
-}
-
 // Static schedule.  Wave w holds units [w uw, (w + 1) uw) (fewer in the last
 // wave), L = their tiles in unit order; it is cut into n = min(P, L / smin)
 // contiguous slices (smin: the shortest slice of a full wave, so that a short
@@ -725,9 +717,9 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
       // of every slot (a slot or stage is reloaded only after its previous
       // copy was consumed, so only the last one can be pending)
       for (int st = 0; st < kS; ++st)
-        if (used_bits & (1u << st)) drain_bar(&s.full[st], ((par_bits >> st) & 1u) ^ 1u, a);
+        if (used_bits & (1u << st)) drain_bar(&s.full[st], ((par_bits >> st) & 1u) ^ 1u);
       for (int sl = 0; sl < kIQ; ++sl)
-        if (qused_bits & (1u << sl)) drain_bar(&s.qfull[sl], ((qpar_bits >> sl) & 1u) ^ 1u, a);
+        if (qused_bits & (1u << sl)) drain_bar(&s.qfull[sl], ((qpar_bits >> sl) & 1u) ^ 1u);
     }
   } else if (warp == 1) {
     // ------------------------------------------------ logits MMA issuer
@@ -783,7 +775,7 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
       }
       if (!ok) {
         mma_commit(&s.drain);
-        drain_bar(&s.drain, 0u, a);
+        drain_bar(&s.drain, 0u);
       }
     }
     __syncwarp();
@@ -832,7 +824,7 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
       }
       if (!ok) {
         mma_commit(&s.drain2);
-        drain_bar(&s.drain2, 0u, a);
+        drain_bar(&s.drain2, 0u);
       }
     }
     __syncwarp();

@@ -101,14 +101,6 @@ __device__ __forceinline__ bool wait_limit(uint64_t* bar, uint32_t parity, const
   return true;
 }
 
-// The same for what this CTA has itself set in motion, after a wait has run out:
-// nothing is recorded.
-__device__ void drain(uint64_t* bar, const ShortArgs& a) {
-  const unsigned long long t0 = now_ns();
-  while (!mbar_try_wait(bar, 0u) && now_ns() - t0 < a.timeout_ns) {
-  }
-}
-
 template <int RP, bool kSelect>
 __global__ void __launch_bounds__(kThreads, 1)
     short_unit_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ, ShortArgs a,
@@ -414,11 +406,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (gave_up) {
     // a wait ran out: the copies and MMAs in flight end (bounded) before this
     // CTA's memory changes hands
-    for (int t = 0; t < logits_issued; ++t) drain(&s.tfull[t], a);
-    if (sums_issued) drain(&s.sigma, a);
-    if (stats_issued) drain(&s.stat, a);
-    for (int t = 0; t < nt; ++t) drain(&s.full[t], a);
-    drain(&s.qfull, a);
+    for (int t = 0; t < logits_issued; ++t) drain_bar(&s.tfull[t], 0u);
+    if (sums_issued) drain_bar(&s.sigma, 0u);
+    if (stats_issued) drain_bar(&s.stat, 0u);
+    for (int t = 0; t < nt; ++t) drain_bar(&s.full[t], 0u);
+    drain_bar(&s.qfull, 0u);
     __syncthreads();
   }
   if (warp == 1) {

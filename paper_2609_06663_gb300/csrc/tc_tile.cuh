@@ -20,6 +20,18 @@ __device__ __forceinline__ unsigned long long now_ns() {
   return t;
 }
 
+// Wait for a first or later phase of an mbarrier that a copy or MMA of this CTA's
+// own completes, after another wait has run out: without regard to the call's
+// limit, which may be shorter than such an operation takes (two seconds, far
+// above any), because what is still in flight when the CTA leaves lands in
+// memory that is no longer its own.
+__device__ __forceinline__ void drain_bar(uint64_t* bar, uint32_t parity) {
+  constexpr unsigned long long kLimitNs = 2000000000ull;
+  const unsigned long long t0 = now_ns();
+  while (!mbar_try_wait(bar, parity) && now_ns() - t0 < kLimitNs) {
+  }
+}
+
 __device__ __forceinline__ uint32_t sw128(int row, int chunk16) {
   return (uint32_t)(row * 128 + ((chunk16 ^ (row & 7)) << 4));
 }

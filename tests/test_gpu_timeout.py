@@ -84,6 +84,29 @@ def test_a_unit_that_gave_up_is_not_finalised():
         assert torch.equal(got[0, 1], ref[0, 1]) and torch.equal(got[1], ref[1])
 
 
+@pytest.mark.parametrize("window", [8, 28], ids=["32_rows", "112_rows"])
+@pytest.mark.parametrize("sched_wave", [0, 4], ids=["default", "schedule"])
+def test_a_limit_shorter_than_a_copy(sched_wave, window):
+    """A limit of a microsecond may run out while the call's own copies and
+    MMAs are in flight; they are waited for with a limit of their own before
+    the memory they land in is given back.  Whether the call makes it or
+    reports the timeout, the calls after it are undisturbed."""
+    w = small_workload(9000, h_kv=2, group=4, window=window, budget=900, dtype="bf16", n_layers=2, clustered=True)
+    K, V, Q = (t.to(DEV) for t in make_inputs(w))
+    p, p_short = (params_of(w, sched_wave=sched_wave, timeout_us=us) for us in (0, 1))
+    want = E.evict(p, K, V, Q, want_scores=True)
+    ws = E.alloc_workspace(p, DEV)
+    for _ in range(10):
+        got = E.evict(p_short, K, V, Q, ws=ws, want_scores=True)
+        status = E.ecokv_device_status(ws)
+        assert status in (E.ECOKV_OK, E.ECOKV_ERR_TIMEOUT)
+        if status == E.ECOKV_OK:
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
+        got = E.evict(p, K, V, Q, ws=ws, want_scores=True)
+        assert E.ecokv_device_status(ws) == E.ECOKV_OK
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
 def test_stall_flag_needs_the_tensor_core_path():
     """The injected stall exists only in the tensor-core kernel; elsewhere the
     flag is refused before anything is launched."""
