@@ -45,8 +45,8 @@
  *    launch per group of at most 120 window rows (128 past 64 MB of keys) when
  *    (h_q / h_kv) * window exceeds that (each group reads K twice); a few short heads (up to 64
  *    window rows, one cluster of CTAs per head holding all its keys, every
- *    head's on the device at once: up to 10240 keys for 7 heads, 5120 for 19,
- *    640 for 152; no variant flag but the centroid's and the MixKV sign, the default
+ *    head's on the device at once: on a GB300 up to 10240 keys for 7 heads, 5120
+ *    for 15, 3840 for 23, 640 for 152; no variant flag but the centroid's and the MixKV sign, the default
  *    schedule) take one kernel that also scores and selects; fp32 inputs,
  *    shorter caches and ECOKV_FLAG_FORCE_SIMT take the CUDA-core passes.  Every path is
  *    deterministic; scores may differ in their last bits between paths and

@@ -12,10 +12,10 @@
 // runs in the same cluster.  One layer of 8 heads x 1024 keys 29.5 -> 20.5 us a
 // call, 4 heads x 5003 keys 40.1 -> 29.5 us.
 //
-// Taken when one cluster per unit fits the device at once (units x CTAs a unit
-// at most the SMs, one CTA an SM) and the window rows are at most 64; a longer
-// grid would run its clusters one after the other with nothing in flight
-// between them, where the persistent kernel streams.
+// Taken when one cluster per unit fits the device at once (one CTA an SM, whole
+// clusters in a GPC: the occupancy query's answer) and the window rows are at
+// most 64; a longer grid would run its clusters one after the other with nothing
+// in flight between them, where the persistent kernel streams.
 //
 // Steps of a CTA (256 threads: two tile groups of four warps, one key per
 // thread; tile t belongs to group t mod 2; four groups measured the same):
@@ -438,7 +438,7 @@ cudaError_t launch_short_rp(const CUtensorMap& tm, const CUtensorMap& tq, const 
     const cudaError_t e = cudaFuncSetAttribute(short_unit_kernel<RP, kSelect>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    // (clusters past 8 are asked for only where max_clusters16 has seen them allowed)
+    // (clusters past 8 are asked for only where clusters_fit has seen them allowed)
     if (cudaFuncSetAttribute(short_unit_kernel<RP, kSelect>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
         cudaSuccess)
       cudaGetLastError();
@@ -462,51 +462,60 @@ cudaError_t launch_short_rp(const CUtensorMap& tm, const CUtensorMap& tq, const 
 }  // namespace
 
 namespace {
-// Clusters of 16 CTAs of this kernel that a device holds at once (an optional
-// size, past the portable 8): 0 = not asked yet, else the number + 1.
-std::atomic<int> g_max16[64];
+// Clusters of C CTAs of this kernel that a device holds at once plus one, at
+// [device][C - 1]; 0 = not asked yet (a racing thread asks again).
+std::atomic<int> g_fit[64][kShortCtas];
 
-int max_clusters16() {
+int clusters_fit(int C) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  int n1 = g_max16[dev].load();
+  int n1 = g_fit[dev][C - 1].load();
   if (n1 == 0) {
     int n = 0;
-    const int smem = (int)sizeof(ShortSmem<64>) + 1024;  // the largest instance
+    const int smem = (int)sizeof(ShortSmem<64>) + 1024;  // the largest instance (each takes an SM for itself)
     const void* k = (const void*)short_unit_kernel<64, true>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-      cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3(16u * 16u, 1, 1);
-      cfg.blockDim = dim3(kThreads, 1, 1);
-      cfg.dynamicSmemBytes = smem;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 16;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) n = 0;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)C * 256u, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        (C > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+        cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+      cudaGetLastError();  // an unavailable configuration leaves no error behind
+      n = 0;
     }
-    cudaGetLastError();  // an unavailable configuration leaves no error behind
     n1 = n + 1;
-    g_max16[dev].store(n1);
+    g_fit[dev][C - 1].store(n1);
   }
   return n1 - 1;
 }
 }  // namespace
 
+// What is resident is the occupancy query's answer, not the SM count's: the SMs
+// of a GPC hold whole clusters only, and a second wave of clusters runs with
+// nothing in flight between them and the first (152 SMs hold 15 clusters of 7 or
+// 8 CTAs, 23 of 6, 28 of 5, 36 of 4, 46 of 3, 76 of 2).
 int short_cluster(int R, int T, long long U, int sms) {
   if (R > 64 || T > kShortTiles * kShortCtas || U > sms) return 0;
-  // eight CTAs a unit (as tiles and SMs allow); past sixteen tiles sixteen
-  // CTAs where every unit's cluster of that size is resident, so that a tile
-  // group has at most two tiles up to 48 of them (4 heads x 5003 keys: 29.0
-  // against 31.0 us a call, and heads of 41 to 80 tiles need them)
+  // past sixteen tiles sixteen CTAs a unit where every unit's cluster of that
+  // size is resident, so that a tile group has at most two tiles up to 48 of
+  // them (4 heads x 5003 keys: 29.0 against 31.0 us a call, and heads of 41 to 80
+  // tiles need them); else eight, as tiles allow, or the most that are resident
+  // for every unit
+  if (T > 16 && U * kShortCtas <= sms && U <= clusters_fit(kShortCtas)) return kShortCtas;
   long long C = sms / U;
   if (C > T) C = T;
-  if (C > 8) C = T > 16 && U <= max_clusters16() ? (C > 16 ? 16 : C) : 8;
-  return C * kShortTiles >= T ? (int)C : 0;
+  if (C > 8) C = 8;
+  for (; C * kShortTiles >= T; --C)
+    if (U <= clusters_fit((int)C)) return (int)C;
+  return 0;
 }
 
 cudaError_t launch_short(const ShortArgs& a, FinalArgs f, int C, cudaStream_t st) {
