@@ -131,11 +131,17 @@ __device__ __forceinline__ float mad_logistic(float dE, float med, float inv) {
   return 1.f / (1.f + expf(-__fmul_rn(__fsub_rn(dE, med), inv)));
 }
 
-// 1 / x in double to about 2^-46: the single-precision reciprocal and one Newton
-// step (a double division takes over 0.5 us here).
-__device__ __forceinline__ double rcp_double(float x) {
-  const double r0 = (double)__frcp_rn(x);
-  return r0 * (2.0 - (double)x * r0);
+// 1 / b for b > 0 (not subnormal) in double, to 2^-46 of it (2^-46.8 measured):
+// one Newton-Raphson step on the single-precision reciprocal of b's mantissa,
+// whose exponent is taken off and put back so that b's whole range is served.
+// Its uses end in single precision, where the scores' errors against 64 bits are
+// those of a division; that would cost a call 0.3 to 1.5 us, double operations
+// being slow here.
+__device__ __forceinline__ double rcp_double(double b) {
+  const int hi = __double2hiint(b), e = (hi & 0x7ff00000) - 0x3ff00000;
+  const double m = __hiloint2double(hi - e, __double2loint(b));  // in [1, 2)
+  const double r0 = (double)__frcp_rn((float)m), r = r0 * (2.0 - m * r0);
+  return __hiloint2double(__double2hiint(r) - e, __double2loint(r));
 }
 
 // Barrier over the cluster (a block barrier when the unit has one CTA), whole
@@ -448,8 +454,10 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
       // raw(j) cnt(j), where cnt(j) = kp except within kp/2 of either end
       float s_raw = sm.red[0][5];
       for (int w = 1; w < Shape<kSh>::kWarps; ++w) s_raw += sm.red[w][5];
-      // (the edge terms as a sum of two floats, exact to 2^-46: a loop in
-      // double takes 1.5 us here)
+      // (the edge terms as a sum of two floats, with the rounding error of every
+      // product (by fma) and sum (Knuth's two-sum) carried along: within 2^-44 at
+      // any pooling width, where the vote sum they are taken from has 24 bits; a
+      // loop in double takes 1.5 us here)
       const int h = hpool;
       float eh = 0.f, el = 0.f;
       auto add = [&](float x, int w) {
@@ -475,7 +483,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
         s_c += sm.red[w][4];
       }
       const double T = (double)Tv;
-      const double sum_sE = ((double)s_de - (double)mnE * T) * rcp_double(denE);
+      const double sum_sE = ((double)s_de - (double)mnE * T) * rcp_double((double)denE);
       const double sum_cs = (double)s_c;
       const double sum_sC = mix ? -sum_cs : (T - sum_cs) * 0.5;
       sm.sc[4] = s_c;
@@ -591,12 +599,7 @@ __device__ __forceinline__ void cluster_unit(const FinalArgs& f, ClusterSmem<kSh
         for (int r = 0; r < C; ++r) sum_imp += sm.simp_all[r];
         dsc0 = (double)f.pool * sum_imp;
       }
-      const float numf = (float)num;
-      sm.sc[5] = 0.f;
-      if (Tv > 0 && numf > 0.f) {
-        const double r0 = (double)__frcp_rn(numf);
-        sm.sc[5] = (float)(dsc0 * (double)denD * (r0 * (2.0 - num * r0)) * rcp_double((float)f.pool));
-      }
+      sm.sc[5] = (Tv > 0 && num > 0.0) ? (float)(dsc0 * (double)denD * rcp_double((double)f.pool * num)) : 0.f;
     }
     __syncthreads();
     const float lamf = sm.sc[0], mnD2 = sm.sc[6], denD = sm.sc[7], scale = sm.sc[5];
