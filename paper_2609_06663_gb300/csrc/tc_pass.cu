@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
           // infinite log-sum-exp and add exactly zero); the statistics
           // columns after them: k . kbar in three terms, k . mu in two
           const uint32_t tb = tl + b * (uint32_t)kNP;
-          float vp[4] = {0.f, 0.f, 0.f, 0.f};
+          float vp[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
           const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
           constexpr int kCW = RP % 32 == 0 ? 32 : (RP % 28 == 0 ? 56 : RP);
 #pragma unroll
@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&s.tmem_empty[b]);
-          const float v = (vp[0] + vp[1]) + (vp[2] + vp[3]);
+          const float v = vote_sum(vp);
           if (sums) {
             const float kkb = (__uint_as_float(st[0]) + __uint_as_float(st[1])) + __uint_as_float(st[2]);
             const float kmu = __uint_as_float(st[3]) + __uint_as_float(st[4]);

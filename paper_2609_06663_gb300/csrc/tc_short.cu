@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int j = 0; j < kMine; ++j) {
       const int t = grp + kGroups * j;
       if (t >= nt) break;
-      float vp[4] = {0.f, 0.f, 0.f, 0.f};
+      float vp[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
 #pragma unroll
       for (int c0 = 0; c0 < RP; c0 += SC::kCW) {
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_landed(rc);
         vote_rows<SC::kCW>(rc, nlse + c0, scale2, vp);
       }
-      const float v = (vp[0] + vp[1]) + (vp[2] + vp[3]);
+      const float v = vote_sum(vp);
       wait(&s.stat, 45u);
       tc_fence_after();
       uint32_t sv[8];

@@ -137,17 +137,22 @@ __device__ __forceinline__ void add_pair(float& x, float& y, float a, float b) {
 }
 
 // The vote of a key: the sum over kN rows of 2^(x scale - lse), x the logits and
-// nlse the negated log2-sum-exp (16-byte aligned).
+// nlse the negated log2-sum-exp (16-byte aligned), in eight partial sums (row c
+// in sum c mod 8).
 template <int kN>
-__device__ __forceinline__ void vote_rows(uint32_t (&rc)[kN], const float* nlse, uint64_t scale2, float (&vp)[4]) {
+__device__ __forceinline__ void vote_rows(uint32_t (&rc)[kN], const float* nlse, uint64_t scale2, float (&vp)[8]) {
 #pragma unroll
   for (int c = 0; c < kN; c += 4) {
     const float4 nl = *reinterpret_cast<const float4*>(nlse + c);
+    const int p = c & 7;
     fma_pair(rc[c], rc[c + 1], scale2, nl.x, nl.y);
     fma_pair(rc[c + 2], rc[c + 3], scale2, nl.z, nl.w);
-    add_pair(vp[0], vp[1], ex2(__uint_as_float(rc[c])), ex2(__uint_as_float(rc[c + 1])));
-    add_pair(vp[2], vp[3], ex2(__uint_as_float(rc[c + 2])), ex2(__uint_as_float(rc[c + 3])));
+    add_pair(vp[p], vp[p + 1], ex2(__uint_as_float(rc[c])), ex2(__uint_as_float(rc[c + 1])));
+    add_pair(vp[p + 2], vp[p + 3], ex2(__uint_as_float(rc[c + 2])), ex2(__uint_as_float(rc[c + 3])));
   }
+}
+__device__ __forceinline__ float vote_sum(const float (&vp)[8]) {
+  return ((vp[0] + vp[1]) + (vp[2] + vp[3])) + ((vp[4] + vp[5]) + (vp[6] + vp[7]));
 }
 
 // Sum of v[j] over the lanes of a warp for every j < N, scattered: five
