@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
             Z = za;
           }
         }
-        if (rs == 0 && r < RP) ust[ustat_lse() + r] = row ? -(M + log2f(Z)) : -INFINITY;
+        if (rs == 0 && r < RP) ust[ustat_lse() + r] = row ? -log2_sum(M, Z) : -INFINITY;
         // kbar in threads 0..63, mu in 64..127
         const float sc = t < 64 ? 1.f / (float)a.kbar_n : 1.f / (float)a.N;
         sx *= sc;

@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float m2 = s.rec[q][2 * kD + r], z2 = s.rec[q][2 * kD + RP + r];
         if (z2 > 0.f) combine_maxsum(M, Z, m2, z2);
       }
-    s.ust[ustat_lse() + r] = r < a.R ? -(M + log2f(Z)) : -INFINITY;
+    s.ust[ustat_lse() + r] = r < a.R ? -log2_sum(M, Z) : -INFINITY;
   }
   fence_proxy_async_smem();
   __syncthreads();

@@ -123,6 +123,18 @@ __device__ __forceinline__ void combine_maxsum(float& m, float& z, float m2, flo
   m = M;
 }
 
+// log2 of a row's sum Z 2^M.  Z is taken against a reference that may lie far
+// below the row's maximum, and a log2 Z of that size is rounded accordingly: its
+// exponent joins M without error (two-sum), so that one rounding of the result is
+// left.
+__device__ __forceinline__ float log2_sum(float M, float Z) {
+  const int b = __float_as_int(Z);
+  const float e = (float)((b >> 23) - 127), f = __int_as_float((b & 0x7fffff) | 0x3f800000);  // Z = 2^e f
+  const float hi = __fadd_rn(M, e), t = __fsub_rn(hi, M);
+  const float lo = __fadd_rn(__fsub_rn(M, __fsub_rn(hi, t)), __fsub_rn(e, t));
+  return __fadd_rn(hi, __fadd_rn(lo, log2f(f)));
+}
+
 // (x, y) <- (x, y) * s + (a, b) as one packed operation, x and y as float bits
 __device__ __forceinline__ void fma_pair(uint32_t& x, uint32_t& y, uint64_t s, float a, float b) {
   const uint64_t r = ffma2((uint64_t)x | (uint64_t)y << 32, s, pack_f32x2(a, b));
