@@ -61,7 +61,7 @@ struct ShortCfg {
   static constexpr int kNQ = (RP + 15) / 16 * 16;  // N of the logits MMA
   static constexpr uint32_t kStatCol = kShortTiles * kNQ;
   static constexpr uint32_t kSigmaCol = kStatCol + 16 * kShortTiles;
-  static_assert(kSigmaCol + 16 <= kTmemCols, "TMEM columns");
+  static_assert(kSigmaCol + 16 * kShortTiles <= kTmemCols, "TMEM columns");
   static constexpr int kCW = RP <= 32 ? RP : (RP == 56 ? 56 : 32);
   static constexpr int kRec = 2 * kD + 2 * RP;     // floats of a record
 };
@@ -204,7 +204,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   fence_proxy_async_smem();
   __syncthreads();
-  // sums of k and k/||k|| over the CTA's keys
+  // sums of k and k/||k|| over each of the CTA's tiles (the tensor core's
+  // accumulation rounds towards zero: a sum that runs on over five tiles has
+  // five times a tile's bias)
   sums_issued = warp == 0 && ok;
   if (sums_issued && elect_one()) {
     tc_fence_after();
@@ -216,8 +218,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint64_t wd0 = smem_desc(wb, 16, wz - wb, 2), wd1 = smem_desc(wb + 1024, 16, wz - wb - 1024, 2);
 #pragma unroll
       for (int k8 = 0; k8 < 8; ++k8)  // 16 keys per step (A: d contiguous)
-        mma_bf16(tmem + SC::kSigmaCol, kd0 + (uint64_t)(t * (kTileBytes >> 4) + k8 * 128),
-                 (k8 < 4 ? wd0 : wd1) + (uint64_t)((k8 & 3) * 2), idesc, (t > 0 || k8 > 0) ? 1u : 0u);
+        mma_bf16(tmem + SC::kSigmaCol + 16u * t, kd0 + (uint64_t)(t * (kTileBytes >> 4) + k8 * 128),
+                 (k8 < 4 ? wd0 : wd1) + (uint64_t)((k8 & 3) * 2), idesc, k8 > 0 ? 1u : 0u);
     }
     mma_commit(&s.sigma);
   }
@@ -249,12 +251,21 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (grp == 0) {
     wait(&s.sigma, 44u);
     tc_fence_after();
-    uint32_t v[4];
-    tmem_ld_x4(tl + SC::kSigmaCol, v);
+    uint32_t v[kShortTiles][4];
+#pragma unroll
+    for (int t = 0; t < kShortTiles; ++t)
+      if (t < nt) tmem_ld_x4(tl + SC::kSigmaCol + 16u * t, v[t]);
     tmem_wait_ld();
     tc_fence_before();
-    mine[kk] = __uint_as_float(v[0]);
-    mine[kD + kk] = (__uint_as_float(v[1]) + __uint_as_float(v[2])) + __uint_as_float(v[3]);
+    float x = 0.f, y = 0.f;
+#pragma unroll
+    for (int t = 0; t < kShortTiles; ++t)
+      if (t < nt) {
+        x += __uint_as_float(v[t][0]);
+        y += (__uint_as_float(v[t][1]) + __uint_as_float(v[t][2])) + __uint_as_float(v[t][3]);
+      }
+    mine[kk] = x;
+    mine[kD + kk] = y;
   }
   __syncthreads();
   if (tid < RP) {
