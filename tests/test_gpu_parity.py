@@ -127,11 +127,13 @@ def test_streaming_schedule_row_groups():
     run_and_compare(w, sched_wave=1, sched_lag=1)
 
 
-def test_streaming_schedule_many_units():
+# (without a schedule asked for, the short-unit kernel takes this shape)
+@pytest.mark.parametrize("wave", [0, 7, 60])
+def test_streaming_schedule_many_units(wave):
     """Sixty heads of 1000 keys (8 tiles): slices that span several heads and
     heads split over several slices."""
     w = small_workload(1000, h_kv=4, group=2, window=4, budget=100, pool_kernel=5, dtype="bf16", n_layers=15)
-    run_and_compare(w, units=[(0, 0), (3, 1), (7, 2), (14, 3)])
+    run_and_compare(w, units=[(0, 0), (3, 1), (7, 2), (14, 3)], sched_wave=wave)
 
 
 @pytest.mark.parametrize("flags,extra", [
@@ -194,8 +196,9 @@ def test_identical_keys_all_ties():
     w = small_workload(n=400, h_kv=1, group=2, window=4, budget=40, dtype="bf16")
     K, V, Q = make_inputs(w)
     K[:] = K[:, :, :1]
-    for flags in (0, E.ECOKV_FLAG_FORCE_SIMT):
-        p = params_of(w, flags=flags)
+    # the short-unit kernel, the streaming kernel (a schedule asked for), the CUDA-core passes
+    for kw in (dict(), dict(sched_wave=1), dict(flags=E.ECOKV_FLAG_FORCE_SIMT)):
+        p = params_of(w, **kw)
         Kd, Vd, Qd = K.to(DEV), V.to(DEV), Q.to(DEV)
         S_g, lam_g, dbg = E.score(p, Kd, Qd, dbg=True)
         idx, Ko, Vo, S, lam = E.evict(p, Kd, Vd, Qd, want_scores=True)
