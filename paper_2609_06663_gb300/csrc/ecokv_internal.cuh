@@ -47,7 +47,7 @@ struct Layout {
                      // (tensor-core passes)
   int p1_stride;     // floats per (unit, chunk) pass-1 partial: 2R + 2D
   int ustat_stride;  // floats per unit statistics record
-  size_t status, sync, p1part, ustat, p2part, simp, dE, cosv, sbuf, norm2;
+  size_t status, sync, p1part, ustat, p2part, simp, dE, cosv, sbuf;
   size_t chosen, src;  // layer-wide budget: chosen positions, gathered rows (U * min(B, N) int32 each)
   size_t lsel;         // layer-wide budget: the layer select's histograms, state and block counts
   size_t vnorm;        // value-norm importance: ||v_i|| of the candidates, U * Tv floats

@@ -909,7 +909,6 @@ __global__ void __launch_bounds__(Cfg<RP>::kThreads, 1)
 }
 
 // per-device host state; a racing thread repeats the idempotent setup
-std::atomic<int> g_num_sms[64];
 std::atomic<bool> g_attr_set[64][8];
 
 template <int RP>
@@ -1008,12 +1007,6 @@ cudaError_t launch_tc(const void* K, const TcArgs& args, cudaStream_t st) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (g_num_sms[dev].load() == 0) {
-    int n = 0;
-    e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    g_num_sms[dev].store(n);
-  }
   CUtensorMap tm, tq;
   e = tc_tensor_maps(K, args.N, args.U, args.Q, args.q_rows, args.RP, &tm, &tq);
   if (e != cudaSuccess) return e;
