@@ -99,28 +99,45 @@ def row_groups(w) -> int:
     return (w.group * w.window + most - 1) // most
 
 
-SMS = 152  # of a GB300
-
-
-def short_units(w) -> bool:
-    """Few short heads take one launch for both passes, scores and selection:
-    up to 64 window rows, one cluster per head, all clusters (at most five
-    tiles of 128 keys a CTA, eight CTAs or, for up to seven heads, sixteen) on
-    the GPU at once."""
-    tiles = (w.n + 127) // 128
-    ctas = min(16 if tiles > 16 and w.units <= 7 else 8, tiles, SMS // w.units)
-    return tensor_path(w) and w.group * w.window <= 64 and 5 * ctas >= tiles
-
-
 def launches_per_call(w) -> int:
-    """Kernels one ecokv_evict call launches: the persistent tensor-core
-    streaming kernel (once per window-row group) or the two CUDA-core passes,
-    then the finalize/select kernel (one thread-block cluster per head, or one
-    CTA per head past 131072 candidates) and the compaction kernel; for a few
-    short heads one kernel in place of the streaming and finalize kernels."""
-    if short_units(w):
-        return 2
+    """Kernels one ecokv_evict call launches where it streams its keys: the
+    persistent tensor-core kernel (once per window-row group) or the two
+    CUDA-core passes, then the finalize/select kernel (one thread-block cluster
+    per head, or one CTA per head past 131072 candidates) and the compaction
+    kernel.  (A few short heads take one kernel in place of the first ones;
+    what a run reports is counted, see kernels_per_call.)"""
     return (row_groups(w) if tensor_path(w) else 2) + 2
+
+
+def kernels_per_call(step) -> int:
+    """Kernels that step(stream) launches: the kernel nodes of the call captured
+    into a CUDA graph, which is not run."""
+    import ctypes
+
+    import torch
+    with open("/proc/self/maps") as f:
+        rt = ctypes.CDLL(next(line.split()[-1] for line in f if "libcudart.so" in line))
+    side = torch.cuda.Stream()
+
+    def ok(code):
+        if code:
+            raise RuntimeError(f"CUDA error {code} while counting the launches of a call")
+
+    graph, n, kind = ctypes.c_void_p(), ctypes.c_size_t(), ctypes.c_int()
+    ok(rt.cudaStreamBeginCapture(ctypes.c_void_p(side.cuda_stream), 2))  # relaxed
+    try:
+        step(side)
+    finally:
+        ok(rt.cudaStreamEndCapture(ctypes.c_void_p(side.cuda_stream), ctypes.byref(graph)))
+    ok(rt.cudaGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    ok(rt.cudaGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    kernels = 0
+    for node in nodes:
+        ok(rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        kernels += kind.value == 0  # cudaGraphNodeTypeKernel
+    ok(rt.cudaGraphDestroy(graph))
+    return kernels
 
 
 # ---------------------------------------------------------------- ranks
@@ -365,7 +382,7 @@ def main():
 
     lb_host = torch.tensor(budgets, dtype=torch.int32) if budgets else None
 
-    def step():
+    def step(stream=stream):
         if adaptive:
             code = E.ecokv_evict_adaptive(p, dt, K, V, Q, idx_a, off_a, Ko_a, Vo_a, lam, ws, ws.numel(), stream)
         elif budgets:
@@ -536,11 +553,7 @@ def main():
                    "evicted_rows_per_s": round(job_rate(world, w.units * max(0, w.n - w.budget), ms_step), 1),
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
-        # the layer-wide budget adds the layer select (3 digits x 2, count, emit) and the split
-        "gpu_launches": (launches_per_call(w) + (9 if adaptive else 0) + (1 if args.variant == "vnorm" else 0)
-                         # the robust forms of Eq. 2: one order-statistics launch
-                         + (1 if args.variant in ("winsor5", "mad") else 0))
-        * args.steps, "clocks": clocks,
+        "gpu_launches": kernels_per_call(step) * args.steps, "clocks": clocks,
         "timing": {"headline": f"{args.steps} steps back to back, CUDA events around the region",
                    "stages": f"{args.steps} further steps with per-launch events (launches serialised)",
                    "staged_ms_per_step": round(staged_ms_step, 5)},
@@ -581,7 +594,7 @@ def run_sweep(args) -> None:
             Vo = torch.empty_like(Ko)
             dt = E.dtype_code(K)
 
-            def step():
+            def step(stream=stream):
                 code = E.ecokv_evict(p, dt, K, V, Q, idx, Ko, Vo, None, None, ws, ws.numel(), stream)
                 if code:
                     raise E.EcokvError(code, "ecokv_evict")
@@ -609,12 +622,14 @@ def run_sweep(args) -> None:
             torch.cuda.synchronize(dev)
             ms = statistics.median(a_.elapsed_time(b_) for a_, b_ in pairs)
             stage_ms = [statistics.median(evs[j].elapsed_time(evs[j + 1]) for evs in stage_ev) for j in range(3)]
+            kernels = kernels_per_call(step)
             bm = byte_model(w)
             gbs = lambda b, t: b / (t * 1e-3) / 1e9
             print(json.dumps({
                 "sweep": "bandwidth sweep (one layer, 8 KV / 32 query heads, bf16, budget 10 %)",
                 "workload": w.name, "n": n, "window": win, "budget": w.budget,
-                "path": (f"tensor-core streaming kernel x{row_groups(w)}" if tensor_path(w) else "CUDA-core passes"),
+                "path": ("CUDA-core passes" if not tensor_path(w) else "short-unit kernel" if kernels == 2 else
+                         f"tensor-core streaming kernel x{kernels - 2}"),
                 "ms_per_call": round(ms, 5), "tokens_per_s": round(w.units * n / (ms * 1e-3), 1),
                 "evicted_rows_per_s": round(w.units * max(0, n - w.budget) / (ms * 1e-3), 1),
                 "alg_gbs": round(gbs(bm["alg"], ms), 1), "bl_gbs": round(gbs(bm["bl"], ms), 1),
