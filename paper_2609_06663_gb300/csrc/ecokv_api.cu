@@ -73,9 +73,13 @@ static ecokv_status check_ws(const ecokv_params* p, void* ws, size_t ws_bytes) {
 }
 
 // Window rows per launch of the tensor-core kernel: all R of a unit up to 120,
-// past that near-equal groups, each of which reads K twice.  Keys past about
-// half of L2 come from DRAM every time, so there a launch takes up to 128 rows
-// (8 heads x 131072 keys, R = 128: 135 us in one launch, 196 in two of 64 rows).
+// past that near-equal groups, each of which reads K twice and folds its own
+// statistics.  Past 64 MB of keys, which then come from DRAM in every read, a
+// launch takes up to 128 rows (8 heads x 131072 keys, R = 128: 135 us of
+// streaming in one launch, 196 in two of 64 rows).  The line bounds what was
+// changed, not what would pay: below it one launch of 128 rows is the shorter one
+// as well (R = 128, us a call, two / one: 4 heads x 1024 47.8 / 34.1, x 8192 60.5
+// / 41.8, x 32768 75.3 / 58.1; 8 heads x 32768, just at it, 95.4 / 75.3).
 static int tc_groups(const ecokv_params& p, int R) {
   const long long key_bytes = (long long)p.n_layers * p.h_kv * p.n * kD * 2;
   const int most = key_bytes > (64LL << 20) ? 128 : 120;

@@ -159,8 +159,8 @@ cudaError_t launch_value_norms(const void* V, ecokv_dtype dt, int U, int N, int 
 bool cluster_finalize_fits(int Tv);
 // k largest of each layer's T scores, ascending positions (layer_select.cu)
 size_t layer_select_scratch_bytes(int n_layers, int T);
-// the order-preserving keys of the ka-th and kb-th largest of each row's
-// T <= 32768 values at out[4 row] and out[4 (rows + row)]; with mad also
+// the order-preserving keys of the ka-th and kb-th largest of each row's T values
+// (1 <= ka, kb <= T <= 2^24) at out[4 row] and out[4 (rows + row)]; with mad also
 // those of |x - m| (m the mean of the first two) at out[4 (2 rows + row)]
 // and out[4 (3 rows + row)] (order_stats.cu)
 cudaError_t launch_order_stats(const float* x, int rows, int T, int ka, int kb, bool mad, unsigned* out,

@@ -5,8 +5,8 @@
 // so one copy beats two trips over the host link); the pass then runs on those
 // copies with V, K_out, V_out and lambda left in host memory, so that the
 // gather reads only the kept V rows over the link and writes the outputs, and
-// the indices made in the workspace, there directly (the indices by a copy of
-// their own: 9 us).  With value-norm importance
+// the indices made in the workspace, there directly (by a copy of their own the
+// indices took 8 us more).  With value-norm importance
 // (ECOKV_FLAG_VNORM_IMP) the norm kernel reads every row of V where it lies,
 // so then all of V crosses the link as well.
 //

@@ -33,7 +33,11 @@ __global__ void __launch_bounds__(Shape<kSh>::kThreads, Shape<kSh>::kMinCtas) fi
 // one an SM: 4 heads x 32768 keys (16 CTAs each) 59.5 / 53.3 / 50.0, 8 x 65536
 // (8 CTAs of 32 candidates a thread) 112 / 99.5 / 90.9, 8 x 8192 38.1 / 35.8 /
 // 35.8; but 8 x 131072, whose clusters of 16 are not all resident at one an SM,
-// 149 / 142 / 158.
+// 149 / 142 / 158.  For its few microseconds nothing that needs shared memory
+// runs beside it on those SMs; a caller with two streams does not notice: two
+// streams of such calls, as used / so, 42.1 / 42.4 us a call at 4 x 32768 and 95.0
+// / 86.7 at 8 x 65536, and four 1024 x 1024 matrix products in the second stream
+// take 28 / 26 and 45 / 30 us longer with a call beside them.
 template <int kSh>
 constexpr int smem_bytes(int spread) {
   const int used = (int)sizeof(ClusterSmem<kSh>), wide = spread == 2 ? 200 * 1024 : (spread == 1 ? 110 * 1024 : 0);

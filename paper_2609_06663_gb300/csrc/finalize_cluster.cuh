@@ -62,7 +62,9 @@ constexpr int kHalo = 16;  // pooling halo kept in shared memory (kernel <= 33)
 // Shapes (kSh), see above: candidates a thread, CTAs a unit, histogram ranges
 // (their 16-bit counts of every rank take the place of the staged scores).
 // Shape 4 is the short-unit kernel's: a CTA's keys are at most 640.  Shape 5 is
-// the small CTA's.
+// the small CTA's.  At the registers that kMinCtas leaves (64; 80 for shape 1, 72
+// for shape 5) the shapes of 32 candidates a thread spill 124 to 132 bytes a
+// thread with the selection and 80 without, shape 5 56 with it.
 template <int kSh>
 struct Shape {
   static constexpr int kThreads = kSh == 5 ? 128 : kCThreads, kWarps = kThreads / 32;

@@ -2,11 +2,11 @@
 // normalisation ablation of Appendix B): the winsorised min-max's clip bounds,
 // and for MAD scaling the median of d_E and the median of |d_E - median|.
 //
-// One CTA per unit: its Tv <= 32768 distances are read in coalesced order
-// into shared memory as order-preserving keys, up to 32 per thread in slots that
-// only it reads, and an MSB-first radix select on the keys finds two ranks at once
-// (longer rows are read from L2 until the keys left under the ranks'
-// prefixes fit those slots, see os_select2_long):
+// One CTA per unit.  Up to 32768 distances are read in coalesced order into
+// shared memory as order-preserving keys, up to 32 per thread in slots that only
+// it reads, and an MSB-first radix select on the keys finds two ranks at once;
+// longer rows are read from L2 until the keys left under the ranks' prefixes fit
+// those slots (os_select2_long):
 // - the row's smallest and largest keys give the prefix every key shares;
 // - one digit of up to 12 bits just below it, counted by direct atomics into
 //   a block-wide histogram (the keys spread over its bins), and a suffix

@@ -95,7 +95,9 @@ struct Cfg {
   // weights; below, the rows leave the tile groups the time
   static constexpr bool kStatNorms = RP > 64;
   // registers a thread: at launch, and after the split between the
-  // warpgroups (tile groups hold a pass-1 sum per row and the columns in work)
+  // warpgroups (tile groups hold a pass-1 sum per row and the columns in work).
+  // Some still spill: 68 to 100 bytes of stores a thread up to 64 rows, 132 past
+  // them (-Xptxas -v); fewer tile-group registers for more elsewhere were slower.
   static constexpr uint32_t kRegsLaunch = RP > 64 ? 128 : 96;
   static constexpr uint32_t kRegsTile = RP > 64 ? 208 : 128, kRegsStats = 56, kRegsCtl = 40;
   static_assert(kTileThreads * kRegsTile + 128 * (kRegsStats + kRegsCtl) <= kThreads * kRegsLaunch &&

@@ -10,7 +10,7 @@
 // and their logits in TMEM through both passes; the pass-1 records go to every
 // CTA by distributed shared memory, and the finalisation (finalize_cluster.cuh)
 // runs in the same cluster.  One layer of 8 heads x 1024 keys 29.5 -> 20.5 us a
-// call, 4 heads x 5003 keys 40.1 -> 29.5 us.
+// call, 4 heads x 5003 keys 40.1 -> 28.7 us.
 //
 // Taken when one cluster per unit fits the device at once (one CTA an SM, whole
 // clusters in a GPC: the occupancy query's answer) and the window rows are at
@@ -519,7 +519,9 @@ int short_cluster(int R, int T, long long U, int sms) {
   // size is resident, so that a tile group has at most two tiles up to 48 of
   // them (4 heads x 5003 keys: 29.0 against 31.0 us a call, and heads of 41 to 80
   // tiles need them); else eight, as tiles allow, or the most that are resident
-  // for every unit
+  // for every unit (56 rows, us a call in two waves / so / by the persistent
+  // kernel: 16 heads x 1019 keys 41.0 / 24.6 / 32.8, 24 x 763 41.0 / 24.6 / 33.1,
+  // 37 x 507 39.0 / 22.6 / 33.1; where nothing fits, 19 x 5115: 55.3 / - / 40.0)
   if (T > 16 && U * kShortCtas <= sms && U <= clusters_fit(kShortCtas)) return kShortCtas;
   long long C = sms / U;
   if (C > T) C = T;
