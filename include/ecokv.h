@@ -43,12 +43,13 @@
  *  - Paths: bf16 inputs with n >= 128 stream K through a persistent
  *    tensor-core kernel, one launch for both of its passes over K, or one
  *    launch per group of at most 120 window rows (128 past 64 MB of keys) when
- *    (h_q / h_kv) * window exceeds that (each group reads K twice); a few short heads (up to 64
- *    window rows, one cluster of CTAs per head holding all its keys, every
- *    head's on the device at once: on a GB300 up to 10240 keys for 7 heads, 5120
- *    for 15, 3840 for 23, 640 for 152; no variant flag but the centroid's and the MixKV sign, the default
- *    schedule) take one kernel that also scores and selects; fp32 inputs,
- *    shorter caches and ECOKV_FLAG_FORCE_SIMT take the CUDA-core passes.  Every path is
+ *    (h_q / h_kv) * window exceeds that (each group reads K twice); a few short
+ *    heads (up to 64 window rows, one cluster of CTAs per head holding all its
+ *    keys, every head's on the device at once: on a GB300 up to 10240 keys for 7
+ *    heads, 5120 for 15, 3840 for 23, 640 for 152; no variant flag but the
+ *    centroid's, the MixKV sign and a lambda override, the default schedule)
+ *    take one kernel that also scores and selects; fp32 inputs, shorter caches
+ *    and ECOKV_FLAG_FORCE_SIMT take the CUDA-core passes.  Every path is
  *    deterministic; scores may differ in their last bits between paths and
  *    between streaming schedules (ecokv_params.sched_*), within the
  *    documented tolerances.
@@ -131,7 +132,8 @@ typedef struct {
                             of every head before any pass 2) */
   int32_t sched_lag;     /* waves between a wave's first and second read of its keys (default 1) */
   uint32_t timeout_us;   /* limit of every bounded device-side wait, microseconds (0 = 2 s); a wait that
-                            runs out records ECOKV_ERR_TIMEOUT in the status word */
+                            runs out records ECOKV_ERR_TIMEOUT in the status word, and the kernel ends
+                            once its own copies and MMAs in flight have (two seconds at most) */
 } ecokv_params;
 
 /* Fill *p with the paper's defaults (Appendix A.3): alpha 0.8, beta 0.6,
